@@ -1636,8 +1636,11 @@ mf_status mf_background_refit(const float *data, int64_t T, int64_t H, int64_t W
             Rinv[i * 6 + j] = -v / R[i * 6 + i];
         }
     }
-    std::vector<float> Q((size_t)T * mf::kRefitBasisPitch, 0.f);
-    double q1[6] = {0};
+    // the workspace's image (basis, R^-1, Q^T 1), sent as one copy
+    std::vector<char> img(mf::refit_workspace(T), 0);
+    float *Q = (float *)(img.data() + mf::refit_q_off());
+    double *q1 = (double *)(img.data() + mf::refit_q1_off(T));
+    std::memcpy(img.data() + mf::refit_rinv_off(T), Rinv, sizeof Rinv);
     for (int64_t t = 0; t < T; t++) {
         const double *f = &phi[(size_t)t * 6];
         for (int j = 0; j < 6; j++) {
@@ -1649,11 +1652,7 @@ mf_status mf_background_refit(const float *data, int64_t T, int64_t H, int64_t W
     }
     cudaStream_t st = (cudaStream_t)stream;
     char *ws = (char *)workspace;
-    cudaError_t e = cudaMemcpyAsync(ws + mf::refit_q_off(), Q.data(), Q.size() * sizeof(float),
-                                    cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(ws + mf::refit_rinv_off(T), Rinv, sizeof Rinv, cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(ws + mf::refit_q1_off(T), q1, sizeof q1, cudaMemcpyHostToDevice, st);
+    const cudaError_t e = cudaMemcpyAsync(ws, img.data(), img.size(), cudaMemcpyHostToDevice, st);
     if (e != cudaSuccess) return fail(MF_ECUDA, "basis upload: %s", cudaGetErrorString(e));
     mf::RefitArgs a{data, T, H, W, scatter, scatter ? n : 0, opts->iterations, (float)opts->delta, resid, coef,
                     ws, stream};

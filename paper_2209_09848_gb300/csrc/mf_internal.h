@@ -378,6 +378,7 @@ struct RefitArgs {
     void *stream;
 };
 constexpr int kRefitBasisPitch = 8;
+constexpr int kRefitMaxResident = 1920;  // frames of the longest series a CTA holds
 size_t refit_workspace(int64_t T);
 // Offsets of the basis pieces in the workspace.
 size_t refit_q_off();

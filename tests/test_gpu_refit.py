@@ -99,3 +99,14 @@ def test_refit_rejects_bad_arguments(mf):
     bad[3, 1] = np.inf
     with pytest.raises(mf.MFError):
         mf.background_refit(D, bad, 1.0, 2)
+
+
+@pytest.mark.parametrize("T", [6, 7, 176, 177, 352, 353, 528, 529, 768, 769, 1152, 1153, 1920, 1921])
+@pytest.mark.parametrize("H,W", [(8, 12), (5, 7)])
+def test_refit_series_lengths(mf, T, H, W):
+    # the edges of the layouts that keep a series on the chip, and the first
+    # length that is re-read from memory; pixel counts that allow 128-bit rows
+    # and one that does not (nor fills a CTA's pixels)
+    from paper_2209_09848_gb300 import synth
+    c = synth.background_case(T, H, W, seed=T, n=3)
+    _check(mf, c, 1.345, 4)
