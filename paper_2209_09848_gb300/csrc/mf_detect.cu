@@ -4,50 +4,58 @@
 // detection per group of touching candidates.
 //
 // Data path, all on the caller's stream, P = H x W pixels:
-//   k_det_cols     thread per (column, chunk of 64 rows): sliding sums over
-//                  the window's rows of the valid scores, their squares and
-//                  the valid count (FP64, FP64, int32 per pixel);
-//   k_det_rows     block per (row, 1024-column tile), row-major: the tile's column sums
+//   k_det_cols     thread per (column, chunk of rows): sliding sums over the
+//                  window's rows of the valid scores, their squares and the
+//                  valid count (FP64, FP64, int32 per pixel);
+//   k_det_rows     block per (row, tile of columns): the tile's column sums
 //                  plus halo in shared memory, prefix sums along the row,
-//                  window sums as prefix differences, then mean, sigma, z,
-//                  the candidate flag and the union-find parent (itself for a
-//                  candidate, -1 otherwise);
+//                  window sums as prefix differences, then z, the candidate
+//                  flag, the union-find parent (itself for a candidate, -1
+//                  otherwise) and the list of candidates;
 //   k_det_union    thread per candidate: union with the candidate neighbours
 //                  above it and to its left (lock-free union-find in which a
 //                  root only ever hangs below a smaller index, so every
 //                  component ends rooted at its smallest flat index);
-//   k_det_flatten  every candidate points at its root;
-//   k_det_peak     per component the largest z (atomicMax on order-
-//                  preserving FP64 bits) and the pixel count; then the
-//                  smallest index attaining that z;
-//   k_det_mark     per root: the peak's FP32 z and root id into a sparse map;
-//   top-k select   the shared radix select and sort (z desc, index asc);
-//   k_det_emit     one record per selected detection and the counts.
+//   k_det_peak_z   every candidate points at its root; per component the
+//                  largest z (atomicMax on order-preserving FP64 bits) and the
+//                  pixel count;
+//   k_det_peak_at  the smallest index attaining that z;
+//   k_det_mark     per root: the peak's FP32 z and index as a selection key;
+//   top-k select   the shared selection over those keys (z desc, index asc);
+//   k_det_emit     one record per selected detection (its window's mean and
+//                  sigma summed again) and the counts.
 // Every reduction is an integer atomic or a fixed-order sum, so reruns are
 // bit-identical.
+//
+// FP64 operations -- arithmetic, comparisons and conversions alike -- issue
+// once per 64 cycles and scheduler on this GPU and bound the first two kernels,
+// so they are counted: conversions go by bits (widen), and k_det_rows keeps
+// FP64 for the sums and the cancelling n s - s1 and n s2 - s1^2, forms z from
+// them in pairs of FP32 numbers, and takes the FP64 formula only for pixels at
+// or above the threshold (or a window near the degenerate limit).
 
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cmath>
 #include <cstdint>
 #include <cstdio>
 
+#include "mf_device.cuh"
 #include "mf_internal.h"
 
 namespace mf {
 namespace {
 
-constexpr int kRowTile = 1024;    // output columns per k_det_rows block
+using dev::sel_key;
+using dev::widen;
+
+constexpr int kRowTile = 2048;  // output columns per k_det_rows block at most
 constexpr int kRowThreads = 256;
 constexpr int kUnionBudget = 1 << 20;  // iterations of one find or merge loop
 
 struct DetectLayout {
-    size_t c1, c2, cn, zd, mean, sd, parent, vsel, ncomp, sel_base, total;
-    // aliases once the window sums are consumed
-    size_t zmax() const { return c1; }                            // P x uint64
-    size_t peak() const { return c2; }                            // P x uint32
-    size_t npix(int64_t P) const { return c2 + (size_t)P * 4; }   // P x int32
-    size_t zsel() const { return cn; }                            // P x float
+    size_t c1, c2, cn, zd, zmax, parent, peak, npix, cand, sel_base, total;
     SelectLayout sel;
 };
 
@@ -62,12 +70,12 @@ DetectLayout detect_layout(int64_t P, int32_t max_out) {
     L.c1 = take((size_t)P * 8);
     L.c2 = take((size_t)P * 8);
     L.cn = take((size_t)P * 4);
-    L.zd = take((size_t)P * 8);
-    L.mean = take((size_t)P * 8);
-    L.sd = take((size_t)P * 8);
+    L.zd = take((size_t)P * 8);    // this and the next five: at candidates only (parent everywhere)
+    L.zmax = take((size_t)P * 8);
     L.parent = take((size_t)P * 4);
-    L.vsel = take((size_t)P * 4);
-    L.ncomp = take(16);
+    L.peak = take((size_t)P * 4);
+    L.npix = take((size_t)P * 4);
+    L.cand = take((size_t)P * 4);  // the candidates' flat indices, in no order
     L.sel_base = off;
     L.sel = select_layout(P, max_out > 0 ? max_out : 1);
     L.total = L.sel_base + L.sel.total;
@@ -80,41 +88,82 @@ __device__ __forceinline__ unsigned long long ord_bits(double v) {
 }
 
 // Vertical window sums: for output row y the rows y - R .. y + R clipped to
-// the image.  A thread owns one column of a chunk of kColChunk output rows:
-// it sums its first row's window directly, then each step adds the row
-// entering the window and drops the row leaving it.
-constexpr int kColChunk = 64;
-__global__ void k_det_cols(const float *__restrict__ s, const int32_t *__restrict__ am, int H, int W, int R,
-                           double *__restrict__ c1, double *__restrict__ c2, int *__restrict__ cn) {
+// the image.  A thread owns one column of a chunk of output rows: it sums its
+// first row's window directly, then each step adds the row entering the window
+// and drops the row leaving it: 4 FP64 operations a pixel plus 2 (2 R + 1) per
+// chunk.  The chunks are as long as two blocks of four warps per SM allow
+// (2048^2, window 255: 108 rows; one block per SM does fewer sums but leaves
+// the pipe idle behind the loads, 132 us).  The count goes by bit masks.
+// Both kernels of the stage, 2048^2 with window 255: 567 -> 236 us.
+__global__ void __launch_bounds__(128) k_det_cols(const float *__restrict__ s, const int32_t *__restrict__ am, int H,
+                                                  int W, int R, int chunk, double *__restrict__ c1,
+                                                  double *__restrict__ c2, int *__restrict__ cn) {
+    constexpr int U = 8;  // rows whose loads are in flight together
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     if (x >= W) return;
-    for (int y0 = blockIdx.y * kColChunk; y0 < H; y0 += gridDim.y * kColChunk) {
-        double a1 = 0.0, a2 = 0.0;
-        int an = 0;
-        auto take = [&](int y, bool add) {
-            if (y < 0 || y >= H) return;
-            const size_t i = (size_t)y * W + x;
-            if (am[i] < 0) return;
-            const double v = (double)s[i];
-            if (add) {
-                a1 += v;
-                a2 += v * v;
-                an += 1;
-            } else {
-                a1 -= v;
-                a2 -= v * v;
-                an -= 1;
+    const int y0 = blockIdx.y * chunk, y1 = min(H, y0 + chunk);
+    double a1 = 0.0, a2 = 0.0;
+    int an = 0;
+    // the valid scores of rows y .. y + U - 1 that lie in lo .. hi - 1, 0
+    // elsewhere, and a bit for each that counts (score and flag are loaded at
+    // once: a score load that waits for its flag would stall the warp)
+    auto fetch = [&](int y, int lo, int hi, float (&v)[U]) {
+        unsigned int bits = 0;
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            const bool in = y + u >= lo && y + u < hi;
+            const size_t i = (size_t)(in ? y + u : 0) * W + x;
+            const int k = am[i];
+            const float f = s[i];
+            const bool ok = in && k >= 0;
+            v[u] = ok ? f : 0.f;
+            bits |= (unsigned int)ok << u;
+        }
+        return bits;
+    };
+    // the rows of the next step are on their way while this one's are summed
+    float vi[U], vo[U], wi[U], wo[U];
+    const int first = max(0, y0 - R - 1), upto = min(H, y0 + R);
+    unsigned int ni, no, mi = fetch(first, first, upto, wi), mo;
+    for (int y = first; y < upto; y += U) {
+        ni = mi;
+#pragma unroll
+        for (int u = 0; u < U; u++) vi[u] = wi[u];
+        mi = fetch(y + U, first, upto, wi);
+        an += __popc(ni);
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            const double d = widen(vi[u]);
+            a1 += d;
+            a2 = fma(d, d, a2);
+        }
+    }
+    mi = fetch(y0 + R, 0, H, wi);
+    mo = fetch(y0 - R - 1, 0, H, wo);
+    for (int y = y0; y < y1; y += U) {
+        ni = mi;
+        no = mo;
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            vi[u] = wi[u];
+            vo[u] = wo[u];
+        }
+        mi = fetch(y + U + R, 0, H, wi);
+        mo = fetch(y + U - R - 1, 0, H, wo);
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            const double di = widen(vi[u]), dn = widen(vo[u]);
+            a1 += di;
+            a2 = fma(di, di, a2);
+            a1 -= dn;
+            a2 = fma(-dn, dn, a2);
+            an += (int)((ni >> u) & 1u) - (int)((no >> u) & 1u);
+            if (y + u < y1) {
+                const size_t i = (size_t)(y + u) * W + x;
+                c1[i] = a1;
+                c2[i] = a2;
+                cn[i] = an;
             }
-        };
-        for (int y = max(0, y0 - R - 1); y < y0 + R && y < H; y++) take(y, true);
-        const int y1 = min(H, y0 + kColChunk);
-        for (int y = y0; y < y1; y++) {
-            take(y + R, true);
-            take(y - R - 1, false);
-            const size_t i = (size_t)y * W + x;
-            c1[i] = a1;
-            c2[i] = a2;
-            cn[i] = an;
         }
     }
 }
@@ -148,23 +197,49 @@ __device__ __forceinline__ T block_exclusive_scan(T v, T *warp_tot) {
     return r;
 }
 
-// Horizontal window sums, statistics, z and the candidate flag for the
-// columns x0 .. x0 + kRowTile - 1 of row y.  Shared entry j holds column
-// lo + j, lo = x0 - R - 1 (0 outside the image); after the prefix scan the
-// window [x - R, x + R] of column x = x0 + t is entries t + 1 .. t + 2R + 1.
+// x = hi + lo to 2^-47 relative, by bits; false where a part could leave the
+// range of normal FP32 numbers.
+__device__ __forceinline__ bool split(double x, float &hi, float &lo) {
+    const uint32_t h = (uint32_t)__double2hiint(x), l = (uint32_t)__double2loint(x);
+    const int e = (int)((h >> 20) & 0x7FFu) - 1023;
+    const bool zero = ((h << 1) | l) == 0u;
+    hi = zero ? 0.f
+              : __uint_as_float((h & 0x80000000u) | (uint32_t)(e + 127) << 23 | ((h & 0xFFFFFu) << 3) | (l >> 29));
+    const float m = (float)(l & 0x1FFFFFFFu) * __uint_as_float((uint32_t)(e + 127 - 52) << 23);
+    lo = zero ? 0.f : ((h & 0x80000000u) ? -m : m);
+    return zero || (e >= -60 && e <= 60);
+}
+
+// The FP64 statistics of one window: mean and variance of n values from their
+// sum and the sum of their squares.
+__device__ __forceinline__ void window_stats(double s1, double s2, int n, double &mean, double &var) {
+    mean = 0.0;
+    var = 0.0;
+    if (n > 0) {
+        const double inv_n = 1.0 / n;
+        mean = s1 * inv_n;
+        var = fmax(s2 * inv_n - mean * mean, 0.0);
+    }
+}
+
+// Horizontal window sums, z and the candidate flag for the columns x0 .. x0 +
+// tile - 1 of row y.  Shared entry j holds column lo + j, lo = x0 - R - 1 (0
+// outside the image); after the prefix scan the window [x - R, x + R] of
+// column x = x0 + t is entries t + 1 .. t + 2R + 1.
 __global__ void __launch_bounds__(kRowThreads) k_det_rows(
     const float *__restrict__ s, const int32_t *__restrict__ am, const double *__restrict__ c1,
-    const double *__restrict__ c2, const int *__restrict__ cn, int H, int W, int R, double thr, int submean,
-    float *__restrict__ z_out, double *__restrict__ zd, double *__restrict__ mean_o, double *__restrict__ sd_o,
-    int *__restrict__ parent) {
+    const double *__restrict__ c2, const int *__restrict__ cn, int H, int W, int R, int tile, double thr,
+    float thr_low, int submean, float *__restrict__ z_out, double *__restrict__ zd,
+    unsigned long long *__restrict__ zmax, unsigned int *__restrict__ peak, int *__restrict__ npix,
+    int *__restrict__ parent, int *__restrict__ cand, SelState *st) {
     extern __shared__ double sm[];
     __shared__ double wt1[kRowThreads / 32], wt2[kRowThreads / 32];
     __shared__ int wtn[kRowThreads / 32];
-    const int tiles = (W + kRowTile - 1) / kRowTile;
+    const int tiles = (W + tile - 1) / tile;
     const int y = (int)(blockIdx.x / tiles);
-    const int x0 = (int)(blockIdx.x % tiles) * kRowTile;
+    const int x0 = (int)(blockIdx.x % tiles) * tile;
     const int lo = x0 - R - 1;
-    const int L = kRowTile + 2 * R + 1;
+    const int L = tile + 2 * R + 1;
     double *p1 = sm;
     double *p2 = sm + L;
     int *pn = reinterpret_cast<int *>(sm + 2 * L);
@@ -177,7 +252,7 @@ __global__ void __launch_bounds__(kRowThreads) k_det_rows(
         pn[j] = in ? cn[row + x] : 0;
     }
     __syncthreads();
-    const int per = (L + blockDim.x - 1) / blockDim.x;
+    const int per = ((L + blockDim.x - 1) / blockDim.x) | 1;  // odd: neighbouring threads on other banks
     const int j0 = min(L, (int)threadIdx.x * per), j1 = min(L, j0 + per);
     double r1 = 0.0, r2 = 0.0;
     int rn = 0;
@@ -198,30 +273,70 @@ __global__ void __launch_bounds__(kRowThreads) k_det_rows(
         pn[j] += on;
     }
     __syncthreads();
-    for (int t = threadIdx.x; t < kRowTile; t += blockDim.x) {
-        const int x = x0 + t;
-        if (x >= W) break;
-        const int n = pn[t + 2 * R + 1] - pn[t];
-        const double s1 = p1[t + 2 * R + 1] - p1[t];
-        const double s2 = p2[t + 2 * R + 1] - p2[t];
-        const size_t i = row + x;
-        double mean = 0.0, var = 0.0, z = 0.0;
-        if (n > 0) {
-            const double inv_n = 1.0 / n;
-            mean = s1 * inv_n;
-            var = fmax(s2 * inv_n - mean * mean, 0.0);
-        }
-        const double sd = sqrt(var);
+    const int lane = threadIdx.x & 31;
+    for (int t0 = threadIdx.x & ~31; t0 < tile; t0 += blockDim.x) {  // whole warps: they add to the list together
+        const int t = t0 + lane, x = x0 + t;
+        const bool in = t < tile && x < W;
+        const size_t i = row + (in ? x : 0);
         bool flag = false;
-        if (am[i] >= 0 && n >= 2 && var > 1e-12 * (mean * mean + var)) {
-            z = ((double)s[i] - (submean ? mean : 0.0)) * rsqrt(var);
-            flag = z > thr;
+        double z = 0.0;
+        if (in) {
+            const bool valid = am[i] >= 0;
+            float zf = 0.f;
+            if (valid) {
+                const int n = pn[t + 2 * R + 1] - pn[t];
+                const double s1 = p1[t + 2 * R + 1] - p1[t];
+                const double s2 = p2[t + 2 * R + 1] - p2[t];
+                // u = n (s - mean) or n s, v = n^2 var: z = u / sqrt(v)
+                const float nf = (float)n;  // n < 2^24
+                const double nd = widen(nf), sd = widen(s[i]);
+                const double u = submean ? fma(nd, sd, -s1) : nd * sd;
+                const double v = fma(nd, s2, -(s1 * s1));
+                float uh, ul, vh, vl, qh, ql;
+                bool plain = split(u, uh, ul);
+                plain = split(v, vh, vl) && plain;
+                plain = split(s2, qh, ql) && plain;
+                plain = plain && n >= 2 && vh > 1e-10f * (nf * qh);  // far from a constant window
+                if (plain) {
+                    // 1 / sqrt(v) = y (1 + e / 2), e = 1 - v y^2 in two FP32 parts
+                    const float y1 = rsqrtf(vh);
+                    const float p = vh * y1, pe = fmaf(vh, y1, -p);
+                    float e = fmaf(-p, y1, 1.f);
+                    e = fmaf(-pe, y1, e);
+                    e = fmaf(-vl * y1, y1, e);
+                    const float yl = 0.5f * e * y1;
+                    const float zh = uh * y1;
+                    float ze = fmaf(uh, y1, -zh);
+                    ze = fmaf(uh, yl, ze);
+                    ze = fmaf(ul, y1, ze);
+                    zf = zh + ze;
+                }
+                if (!plain || !(zf < thr_low)) {
+                    double mean, var;
+                    window_stats(s1, s2, n, mean, var);
+                    if (n >= 2 && var > 1e-12 * (mean * mean + var)) {
+                        z = ((double)s[i] - (submean ? mean : 0.0)) * rsqrt(var);
+                        flag = z > thr;
+                    }
+                    zf = (float)z;
+                }
+            }
+            if (z_out) z_out[i] = zf;
+            parent[i] = flag ? (int)i : -1;
+            if (flag) {
+                zd[i] = z;
+                zmax[i] = 0ull;
+                peak[i] = 0xFFFFFFFFu;
+                npix[i] = 0;
+            }
         }
-        zd[i] = z;
-        mean_o[i] = mean;
-        sd_o[i] = sd;
-        if (z_out) z_out[i] = (float)z;
-        parent[i] = flag ? (int)i : -1;
+        const unsigned int m = __ballot_sync(0xffffffffu, flag);
+        if (m) {
+            unsigned int at = 0;
+            if (lane == 0) at = atomicAdd(&st->ticket, (unsigned int)__popc(m));
+            at = __shfl_sync(0xffffffffu, at, 0);
+            if (flag) cand[at + __popc(m & ((1u << lane) - 1u))] = (int)i;
+        }
     }
 }
 
@@ -255,80 +370,107 @@ __device__ __forceinline__ void uf_merge(int *parent, int a, int b, int *status)
     atomicCAS(status, 0, 3);
 }
 
-__global__ void k_det_union(int *__restrict__ parent, int H, int W, int *status) {
-    const int64_t P = (int64_t)H * W;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < P; i += (int64_t)gridDim.x * blockDim.x) {
-        if (parent[i] < 0) continue;
-        const int y = (int)(i / W), x = (int)(i % W);
-        const int me = (int)i;
-        if (x > 0 && parent[i - 1] >= 0) uf_merge(parent, me, me - 1, status);
+// The kernels below walk the list of candidates, st->ticket of them.
+__global__ void k_det_union(int *__restrict__ parent, const int *__restrict__ cand, const SelState *st, int W,
+                            int *status) {
+    const unsigned int n = st->ticket;
+    for (unsigned int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) {
+        const int i = cand[j];
+        const int y = i / W, x = i % W;
+        if (x > 0 && parent[i - 1] >= 0) uf_merge(parent, i, i - 1, status);
         if (y > 0) {
-            const int64_t up = i - W;
-            if (x > 0 && parent[up - 1] >= 0) uf_merge(parent, me, (int)(up - 1), status);
-            if (parent[up] >= 0) uf_merge(parent, me, (int)up, status);
-            if (x + 1 < W && parent[up + 1] >= 0) uf_merge(parent, me, (int)(up + 1), status);
+            const int up = i - W;
+            if (x > 0 && parent[up - 1] >= 0) uf_merge(parent, i, up - 1, status);
+            if (parent[up] >= 0) uf_merge(parent, i, up, status);
+            if (x + 1 < W && parent[up + 1] >= 0) uf_merge(parent, i, up + 1, status);
         }
     }
 }
 
-__global__ void k_det_flatten(int *__restrict__ parent, int64_t P, int *status) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < P; i += (int64_t)gridDim.x * blockDim.x)
-        if (parent[i] >= 0) parent[i] = uf_find(parent, (int)i, status);
-}
-
-__global__ void k_det_peak_z(const int *__restrict__ parent, const double *__restrict__ zd, int64_t P,
-                             unsigned long long *__restrict__ zmax, int *__restrict__ npix) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < P; i += (int64_t)gridDim.x * blockDim.x) {
-        const int r = parent[i];
-        if (r < 0) continue;
+__global__ void k_det_peak_z(int *parent, const int *__restrict__ cand, const SelState *st,
+                             const double *__restrict__ zd, unsigned long long *__restrict__ zmax,
+                             int *__restrict__ npix, int *status) {
+    const unsigned int n = st->ticket;
+    for (unsigned int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) {
+        const int i = cand[j];
+        const int r = uf_find(parent, i, status);
+        parent[i] = r;  // others that pass through i meet an ancestor either way
         atomicMax(zmax + r, ord_bits(zd[i]));
         atomicAdd(npix + r, 1);
     }
 }
 
-__global__ void k_det_peak_at(const int *__restrict__ parent, const double *__restrict__ zd, int64_t P,
-                              const unsigned long long *__restrict__ zmax, unsigned int *__restrict__ peak) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < P; i += (int64_t)gridDim.x * blockDim.x) {
-        const int r = parent[i];
-        if (r < 0) continue;
+__global__ void k_det_peak_at(const int *__restrict__ parent, const int *__restrict__ cand, const SelState *st,
+                              const double *__restrict__ zd, const unsigned long long *__restrict__ zmax,
+                              unsigned int *__restrict__ peak) {
+    const unsigned int n = st->ticket;
+    for (unsigned int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) {
+        const int i = cand[j], r = parent[i];
         if (ord_bits(zd[i]) == zmax[r]) atomicMin(peak + r, (unsigned int)i);
     }
 }
 
-__global__ void k_det_mark(const int *__restrict__ parent, const double *__restrict__ zd, int64_t P,
-                           const unsigned int *__restrict__ peak, float *__restrict__ zsel, int *__restrict__ vsel,
-                           int *ncomp) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < P; i += (int64_t)gridDim.x * blockDim.x) {
-        if (parent[i] != (int)i) continue;
-        const unsigned int pk = peak[i];
-        zsel[pk] = (float)zd[pk];
-        vsel[pk] = (int)i;
-        atomicAdd(ncomp, 1);
+__global__ void k_det_mark(const int *__restrict__ parent, const int *__restrict__ cand, SelState *st,
+                           const double *__restrict__ zd, const unsigned int *__restrict__ peak,
+                           unsigned long long *__restrict__ keys) {
+    const unsigned int n = st->ticket;
+    const unsigned int lane = threadIdx.x & 31;
+    for (unsigned int j0 = blockIdx.x * blockDim.x + (threadIdx.x & ~31u); j0 < n; j0 += gridDim.x * blockDim.x) {
+        const int i = j0 + lane < n ? cand[j0 + lane] : -1;
+        const bool root = i >= 0 && parent[i] == i;
+        const unsigned int m = __ballot_sync(0xffffffffu, root);
+        if (m == 0) continue;
+        unsigned int at = 0;
+        if (lane == 0) at = atomicAdd(&st->list, (unsigned int)__popc(m));
+        at = __shfl_sync(0xffffffffu, at, 0);
+        if (root) {
+            const unsigned int pk = peak[i];
+            keys[at + __popc(m & ((1u << lane) - 1u))] = sel_key((float)zd[pk], pk);
+        }
     }
 }
 
-__global__ void k_det_emit(const unsigned long long *__restrict__ top, const SelState *st, int max_out,
-                           const int *__restrict__ vsel, const float *__restrict__ s, const int32_t *__restrict__ am,
-                           const double *__restrict__ zd, const double *__restrict__ mean_o,
-                           const double *__restrict__ sd_o, const int *__restrict__ npix, int W, const int *ncomp,
-                           mf_detection *__restrict__ out, int32_t *__restrict__ n_out) {
-    const int n = st ? (int)min(st->count, (unsigned int)max_out) : 0;
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i == 0) {
-        n_out[0] = *ncomp;
+// A warp per detection; its lanes sum the peak's window again from the column
+// sums of the peak's row.
+__global__ void __launch_bounds__(256) k_det_emit(
+    const unsigned long long *__restrict__ top, const SelState *st, int max_out, const int *__restrict__ parent,
+    const float *__restrict__ s, const int32_t *__restrict__ am, const double *__restrict__ zd,
+    const double *__restrict__ c1, const double *__restrict__ c2, const int *__restrict__ cn,
+    const int *__restrict__ npix, int W, int R, mf_detection *__restrict__ out, int32_t *__restrict__ n_out) {
+    const int n = max_out > 0 ? (int)st->count : 0;
+    const int i = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        n_out[0] = (int32_t)st->list;
         n_out[1] = n;
     }
     if (i >= n) return;
-    const unsigned long long key = top[i];
-    const int p = (int)(0xFFFFFFFFu - (unsigned int)(key & 0xFFFFFFFFull));
+    const int p = (int)(0xFFFFFFFFu - (unsigned int)(top[i] & 0xFFFFFFFFull));
+    const int y = p / W, x = p % W;
+    double s1 = 0.0, s2 = 0.0;
+    int cnt = 0;
+    for (int q = max(0, x - R) + lane; q <= min(W - 1, x + R); q += 32) {
+        const size_t at = (size_t)y * W + q;
+        s1 += c1[at];
+        s2 += c2[at];
+        cnt += cn[at];
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        s1 += __shfl_xor_sync(0xffffffffu, s1, o);
+        s2 += __shfl_xor_sync(0xffffffffu, s2, o);
+        cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
+    }
+    if (lane != 0) return;
+    double mean, var;
+    window_stats(s1, s2, cnt, mean, var);
     mf_detection d;
-    d.y = p / W;
-    d.x = p % W;
+    d.y = y;
+    d.x = x;
     d.k = am[p];
-    d.npix = npix[vsel[p]];
+    d.npix = npix[parent[p]];
     d.z = zd[p];
-    d.mean = mean_o[p];
-    d.sigma = sd_o[p];
+    d.mean = mean;
+    d.sigma = sqrt(var);
     d.snr = s[p];
     d.reserved = 0;
     out[i] = d;
@@ -336,7 +478,7 @@ __global__ void k_det_emit(const unsigned long long *__restrict__ top, const Sel
 
 int grid_for(int64_t n, int threads) {
     const int64_t b = (n + threads - 1) / threads;
-    return (int)(b < 152 * 32 ? (b < 1 ? 1 : b) : 152 * 32);
+    return (int)(b < 152 * 8 ? (b < 1 ? 1 : b) : 152 * 8);
 }
 
 struct Scope {
@@ -360,15 +502,15 @@ int launch_detect(const DetectArgs &a, char *err, size_t errlen) {
     double *c2 = reinterpret_cast<double *>(ws + L.c2);
     int *cn = reinterpret_cast<int *>(ws + L.cn);
     double *zd = reinterpret_cast<double *>(ws + L.zd);
-    double *mean = reinterpret_cast<double *>(ws + L.mean);
-    double *sd = reinterpret_cast<double *>(ws + L.sd);
+    unsigned long long *zmax = reinterpret_cast<unsigned long long *>(ws + L.zmax);
     int *parent = reinterpret_cast<int *>(ws + L.parent);
-    int *vsel = reinterpret_cast<int *>(ws + L.vsel);
-    int *ncomp = reinterpret_cast<int *>(ws + L.ncomp);
-    unsigned long long *zmax = reinterpret_cast<unsigned long long *>(ws + L.zmax());
-    unsigned int *peak = reinterpret_cast<unsigned int *>(ws + L.peak());
-    int *npix = reinterpret_cast<int *>(ws + L.npix(P));
-    float *zsel = reinterpret_cast<float *>(ws + L.zsel());
+    unsigned int *peak = reinterpret_cast<unsigned int *>(ws + L.peak);
+    int *npix = reinterpret_cast<int *>(ws + L.npix);
+    int *cand = reinterpret_cast<int *>(ws + L.cand);
+    char *sws = ws + L.sel_base;
+    SelState *st = reinterpret_cast<SelState *>(sws + L.sel.st_off);
+    unsigned long long *keys = reinterpret_cast<unsigned long long *>(sws + L.sel.keys_off);
+    const unsigned long long *top = reinterpret_cast<const unsigned long long *>(sws + L.sel.top_off);
     int *status = status_word(err, errlen);
     if (!status) return (int)cudaErrorUnknown;
     cudaError_t e;
@@ -380,60 +522,56 @@ int launch_detect(const DetectArgs &a, char *err, size_t errlen) {
             return (int)e;                                                       \
         }                                                                        \
     } while (0)
-    {
-        Scope sc(kKDetStats, stream);
-        const dim3 grid((unsigned)((W + 127) / 128), (unsigned)std::min(65535, (H + kColChunk - 1) / kColChunk));
-        k_det_cols<<<grid, 128, 0, stream>>>(a.snr_max, a.argmax, H, W, R, c1, c2, cn);
-    }
-    DET_CHECK("k_det_cols");
-    {
-        const size_t smem = (size_t)(kRowTile + 2 * R + 1) * (8 + 8 + 4);
-        e = cudaFuncSetAttribute(k_det_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) {
-            snprintf(err, errlen, "cudaFuncSetAttribute(k_det_rows): %s", cudaGetErrorString(e));
-            return (int)e;
-        }
-        Scope sc(kKDetStats, stream);
-        const unsigned grid = (unsigned)(((W + kRowTile - 1) / kRowTile) * (int64_t)H);
-        k_det_rows<<<grid, kRowThreads, smem, stream>>>(a.snr_max, a.argmax, c1, c2, cn, H, W, R, a.threshold,
-                                                        a.subtract_mean, a.z_out, zd, mean, sd, parent);
-    }
-    DET_CHECK("k_det_rows");
-    // the window sums are consumed: their space holds the per-root maxima,
-    // peaks and counts from here on
-    e = cudaMemsetAsync(zmax, 0, (size_t)P * 8, stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(peak, 0xFF, (size_t)P * 4, stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(npix, 0, (size_t)P * 4, stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(vsel, 0xFF, (size_t)P * 4, stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(ncomp, 0, 16, stream);
+    e = cudaMemsetAsync(st, 0, sizeof(SelState), stream);
     if (e != cudaSuccess) {
         snprintf(err, errlen, "cudaMemsetAsync: %s", cudaGetErrorString(e));
         return (int)e;
     }
     {
+        // two blocks of four warps per SM, but no chunk shorter than 8 rows
+        const int nbx = (W + 127) / 128, chunks = std::max(1, 2 * 152 / nbx);
+        const int chunk = std::max({8, (H + chunks - 1) / chunks, (H + 65534) / 65535});
+        const dim3 grid((unsigned)nbx, (unsigned)((H + chunk - 1) / chunk));
+        Scope sc(kKDetStats, stream);
+        k_det_cols<<<grid, 128, 0, stream>>>(a.snr_max, a.argmax, H, W, R, chunk, c1, c2, cn);
+    }
+    DET_CHECK("k_det_cols");
+    {
+        const int tile = std::min(kRowTile, (W + 31) / 32 * 32);
+        const size_t smem = (size_t)(tile + 2 * R + 1) * (8 + 8 + 4);
+        e = cudaFuncSetAttribute(k_det_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) {
+            snprintf(err, errlen, "cudaFuncSetAttribute(k_det_rows): %s", cudaGetErrorString(e));
+            return (int)e;
+        }
+        // below this an FP32 z (good to 1e-6) cannot belong to a candidate
+        const double low = a.threshold - 1e-5 * std::max(1.0, std::fabs(a.threshold));
+        const float thr_low = (float)std::max(-3e38, std::min(3e38, low));
+        Scope sc(kKDetStats, stream);
+        const unsigned grid = (unsigned)(((W + tile - 1) / tile) * (int64_t)H);
+        k_det_rows<<<grid, kRowThreads, smem, stream>>>(a.snr_max, a.argmax, c1, c2, cn, H, W, R, tile, a.threshold,
+                                                        thr_low, a.subtract_mean, a.z_out, zd, zmax, peak, npix,
+                                                        parent, cand, st);
+    }
+    DET_CHECK("k_det_rows");
+    {
         Scope sc(kKDetComponents, stream);
         const int g = grid_for(P, 256);
-        k_det_union<<<g, 256, 0, stream>>>(parent, H, W, status);
-        k_det_flatten<<<g, 256, 0, stream>>>(parent, P, status);
-        k_det_peak_z<<<g, 256, 0, stream>>>(parent, zd, P, zmax, npix);
-        k_det_peak_at<<<g, 256, 0, stream>>>(parent, zd, P, zmax, peak);
-        k_det_mark<<<g, 256, 0, stream>>>(parent, zd, P, peak, zsel, vsel, ncomp);
+        k_det_union<<<g, 256, 0, stream>>>(parent, cand, st, W, status);
+        k_det_peak_z<<<g, 256, 0, stream>>>(parent, cand, st, zd, zmax, npix, status);
+        k_det_peak_at<<<g, 256, 0, stream>>>(parent, cand, st, zd, zmax, peak);
+        k_det_mark<<<g, 256, 0, stream>>>(parent, cand, st, zd, peak, keys);
     }
     DET_CHECK("k_det components");
-    const SelState *sst = nullptr;
-    const unsigned long long *top = nullptr;
     if (a.max_out > 0) {
-        char *sws = ws + L.sel_base;
-        const int rc = launch_select(zsel, vsel, P, a.max_out, sws, L.sel, stream, err, errlen);
+        const int rc = launch_select_list(P, a.max_out, 0, sws, L.sel, stream, err, errlen);
         if (rc) return rc;
-        sst = reinterpret_cast<const SelState *>(sws + L.sel.st_off);
-        top = reinterpret_cast<const unsigned long long *>(sws + L.sel.top_off);
     }
     {
         Scope sc(kKDetEmit, stream);
         const int n = a.max_out > 0 ? a.max_out : 1;
-        k_det_emit<<<(n + 255) / 256, 256, 0, stream>>>(top, sst, a.max_out, vsel, a.snr_max, a.argmax, zd, mean,
-                                                        sd, npix, W, ncomp, a.out, a.n_out);
+        k_det_emit<<<(n + 7) / 8, 256, 0, stream>>>(top, st, a.max_out, parent, a.snr_max, a.argmax, zd, c1, c2, cn,
+                                                    npix, W, R, a.out, a.n_out);
     }
     DET_CHECK("k_det_emit");
 #undef DET_CHECK

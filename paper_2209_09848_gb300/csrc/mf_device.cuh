@@ -103,5 +103,24 @@ __device__ __forceinline__ unsigned long long pack_key(float snr, int k) {
     return ((unsigned long long)b << 32) | (unsigned long long)(0xFFFFFFFFu - (uint32_t)k);
 }
 
+// Selection key: larger score first, then smaller index; unique per index.
+__device__ __forceinline__ unsigned long long sel_key(float score, uint32_t i) {
+    uint32_t b = __float_as_uint(score);
+    b = (b & 0x80000000u) ? ~b : (b | 0x80000000u);
+    return ((unsigned long long)b << 32) | (unsigned long long)(0xFFFFFFFFu - i);
+}
+
+// An FP32 value as FP64, by its bits: a conversion instruction costs an FP64
+// operation (1/64 of the FP32 rate on this GPU).  Exact for every value:
+// subnormals are scaled by 2^64 first, infinities and NaN keep their exponent.
+__device__ __forceinline__ double widen(float v) {
+    const uint32_t b = __float_as_uint(v), m = b & 0x7FFFFFFFu;
+    const bool small = m < 0x00800000u;
+    const uint32_t n = small ? __float_as_uint(__uint_as_float(m) * 18446744073709551616.f) : m;
+    const uint32_t off = small ? 0x38000000u - (64u << 20) : (m >= 0x7F800000u ? 0x70000000u : 0x38000000u);
+    const uint32_t hi = n ? (n >> 3) + off : 0u;
+    return __hiloint2double((int)(hi | (b & 0x80000000u)), (int)(n << 29));
+}
+
 }  // namespace dev
 }  // namespace mf

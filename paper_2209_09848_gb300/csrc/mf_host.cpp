@@ -536,13 +536,14 @@ struct HostLayouts {
     std::vector<mf::DenBox> boxes;
     std::vector<int32_t> run_off;
     std::vector<float> wts;
+    std::vector<double> wts64;
 };
 
 size_t layout_bytes(const mf_prf_table *t, const HostLayouts &h) {
     return h.blocks.size() + h.hdr.size() * sizeof(mf::FrameHdr) + t->plan.members.size() * sizeof(int32_t) +
            h.segs.size() * sizeof(int32_t) + t->plan.seg_ref.size() * sizeof(int32_t) +
            h.runs.size() * sizeof(mf::RunRec) + h.boxes.size() * sizeof(mf::DenBox) +
-           h.run_off.size() * sizeof(int32_t) + h.wts.size() * sizeof(float) + t->taps.size() * sizeof(double) +
+           h.run_off.size() * sizeof(int32_t) + h.wts.size() * (sizeof(float) + sizeof(double)) + t->taps.size() * sizeof(double) +
            t->shifts.size() * sizeof(int32_t);
 }
 
@@ -746,6 +747,7 @@ void denominator_layouts(mf_prf_table *t, HostLayouts &out) {
     std::vector<mf::RunRec> runs;
     std::vector<int32_t> run_off(K + 1, 0);
     std::vector<float> wts;
+    std::vector<double> wts64;
     int64_t nnz_total = 0;
     std::vector<double> dense;
     std::vector<char> hit;
@@ -767,7 +769,6 @@ void denominator_layouts(mf_prf_table *t, HostLayouts &out) {
                         size_t n) {
             const int32_t x0 = (int32_t)(4 * floor_div(xfirst, 4));
             const int32_t nch = (int32_t)((xlast - x0 + 1 + 3) / 4);
-            while (wts.size() % 4) wts.push_back(0.f);
             mf::RunRec r;
             r.dy = row;
             r.x0 = x0;
@@ -775,7 +776,12 @@ void denominator_layouts(mf_prf_table *t, HostLayouts &out) {
             r.woff = (int32_t)wts.size();
             const size_t base = wts.size();
             wts.resize(base + (size_t)nch * 4, 0.f);
-            for (size_t q = 0; q < n; q++) wts[base + (col ? col[q] : xfirst + (int32_t)q) - x0] = (float)val[q];
+            wts64.resize(wts.size(), 0.0);
+            for (size_t q = 0; q < n; q++) {
+                const size_t at = base + (col ? col[q] : xfirst + (int32_t)q) - x0;
+                wts64[at] = val[q];
+                wts[at] = (float)val[q];
+            }
             runs.push_back(r);
         };
         if (bw * bh <= (int64_t)100 * T + 4096) {
@@ -881,6 +887,7 @@ void denominator_layouts(mf_prf_table *t, HostLayouts &out) {
     out.runs = std::move(runs);
     out.run_off = std::move(run_off);
     out.wts = std::move(wts);
+    out.wts64 = std::move(wts64);
 }
 
 mf_status finish_table(mf_prf_table *t) {
@@ -899,6 +906,7 @@ mf_status finish_table(mf_prf_table *t) {
     blk.add(&t->d_boxes, h.boxes.data(), h.boxes.size());
     blk.add(&t->d_run_off, h.run_off.data(), h.run_off.size());
     blk.add(&t->d_wts, h.wts.data(), h.wts.size());
+    blk.add(&t->d_wts64, h.wts64.data(), h.wts64.size());
     blk.add(&t->d_taps64, t->taps.data(), t->taps.size());
     blk.add(&t->d_shifts, t->shifts.data(), t->shifts.size());
     if ((s = blk.upload(&t->d_mem, &t->d_mem_pooled)) != MF_OK) return s;
@@ -953,6 +961,7 @@ void free_device(mf_prf_table *t) {
     t->d_boxes = nullptr;
     t->d_run_off = nullptr;
     t->d_wts = nullptr;
+    t->d_wts64 = nullptr;
     t->d_taps64 = nullptr;
     t->d_shifts = nullptr;
 }

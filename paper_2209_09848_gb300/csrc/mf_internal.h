@@ -259,6 +259,7 @@ struct mf_prf_table {
     size_t den_smem = 0;                 // its dynamic shared memory
     int32_t *d_run_off = nullptr;        // [K + 1]
     float *d_wts = nullptr;              // run weights
+    double *d_wts64 = nullptr;           // the same in FP64 (re-score)
     double *d_taps64 = nullptr;          // [K][T][25]
     int32_t *d_shifts = nullptr;         // [K][T][2]
 };
@@ -324,19 +325,21 @@ struct RescoreArgs {
 };
 size_t rescore_workspace(int64_t H, int64_t W, int32_t k_top);
 
-// Top-k selection by a float score (mf_kernels.cu): among pixels with
+// Top-k selection by a float score (mf_select.cu): among pixels with
 // valid[i] >= 0, the k_top largest keys (order-preserving score bits << 32 |
 // (0xFFFFFFFF - i)), i.e. score descending then index ascending, sorted
 // descending into the `top` slice of the workspace.  P < 2^32, k_top <=
 // kMaxTop.
 constexpr int kMaxTop = 16384;
+constexpr int kSelFirstBits = 15;  // key bits of the first histogram over a map
 struct SelState {
-    unsigned long long prefix;  // selected high bits so far
-    unsigned long long thresh;  // final k_top-th largest key (0: take every valid key)
-    unsigned int need;          // keys still to take at and below the current prefix
-    unsigned int total;         // valid keys
-    unsigned int count;         // compacted keys
-    unsigned int pad;
+    unsigned long long prefix;  // high bits fixed so far; keys below are out
+    unsigned int need;          // keys wanted among those that share the prefix
+    unsigned int list;          // keys in the list
+    unsigned int n;             // keys to rank
+    unsigned int refined;       // they stand in the refined list, not the first
+    unsigned int count;         // keys selected: min(k_top, valid keys)
+    unsigned int ticket;        // blocks of the histogram that have finished
 };
 struct SelectLayout {
     size_t keys_off, hist_off, st_off, top_off, total;
@@ -344,6 +347,10 @@ struct SelectLayout {
 SelectLayout select_layout(int64_t P, int32_t k_top);
 int launch_select(const float *score, const int32_t *valid, int64_t P, int32_t k_top, char *ws,
                   const SelectLayout &L, void *stream, char *err, size_t errlen);
+// The same from a list of keys already in the workspace's keys slice, with its
+// length in SelState.list and the rest of SelState clear (fixed_bits = 0).
+int launch_select_list(int64_t P, int32_t k_top, int fixed_bits, char *ws, const SelectLayout &L, void *stream,
+                       char *err, size_t errlen);
 int launch_rescore(const RescoreArgs &a, char *err, size_t errlen);
 
 // Score normalisation and candidate extraction (mf_detect.cu).

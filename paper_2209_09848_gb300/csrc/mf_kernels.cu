@@ -22,6 +22,7 @@
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
+#include <climits>
 #include <cstdio>
 #include <type_traits>
 #include <algorithm>
@@ -1383,185 +1384,11 @@ int batch_enqueue(BatchDevice *b, const SearchArgs *items, int n, void *stream_v
 // ------------------------------------------------------------ rescore ---
 //
 // Candidate list (Section 3.3: scores above a threshold are candidates) and
-// FP64 re-score.  Candidates are ranked by a unique 64-bit key, (order-
-// preserving SNR bits << 32) | (0xFFFFFFFF - flat index): descending key =
-// SNR descending, then flat index ascending.  A 4-pass radix select over 16
-// bits at a time finds the k_top-th largest key, a compaction keeps the keys
-// at or above it, one CTA sorts them, and one warp per candidate recomputes
-// N and D in FP64 from the master stack.
+// FP64 re-score: the k_top best start pixels (mf_select.cu), then N and D of
+// each in FP64 from the master stack.
 
 namespace {
 
-__global__ void k_sel_keys(const float *__restrict__ snr_max, const int32_t *__restrict__ argmax, int64_t P,
-                           unsigned long long *__restrict__ keys, unsigned int *__restrict__ hist,
-                           SelState *st) {
-    // the block's bins in a shared-memory table (open addressing, bin ->
-    // count), flushed into the global histogram with one add per distinct
-    // bin: a score map's keys fall in few bins, which global atomics from
-    // every pixel would serialise on; a bin that finds the table full is
-    // added globally at once
-    constexpr int kSlots = 1024;
-    constexpr unsigned int kEmpty = 0xFFFFFFFFu;
-    __shared__ unsigned int slot_bin[kSlots], slot_cnt[kSlots];
-    for (int j = threadIdx.x; j < kSlots; j += blockDim.x) {
-        slot_bin[j] = kEmpty;
-        slot_cnt[j] = 0u;
-    }
-    __syncthreads();
-    unsigned int valid = 0;  // keys this thread made; summed per warp into st->total
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < P; i += (int64_t)gridDim.x * blockDim.x) {
-        unsigned long long key = 0ull;
-        if (argmax[i] >= 0) {
-            uint32_t b = __float_as_uint(snr_max[i]);
-            b = (b & 0x80000000u) ? ~b : (b | 0x80000000u);
-            key = ((unsigned long long)b << 32) | (unsigned long long)(0xFFFFFFFFu - (uint32_t)i);
-            valid++;
-            const unsigned int bin = (unsigned int)(key >> 48);
-            unsigned int h = (bin * 2654435761u) >> 22;  // 10 bits
-            bool added = false;
-            for (int probe = 0; probe < kSlots; probe++, h = (h + 1) & (kSlots - 1)) {
-                const unsigned int old = atomicCAS(&slot_bin[h], kEmpty, bin);
-                if (old == kEmpty || old == bin) {
-                    atomicAdd(&slot_cnt[h], 1u);
-                    added = true;
-                    break;
-                }
-            }
-            if (!added) atomicAdd(&hist[bin], 1u);
-        }
-        keys[i] = key;
-    }
-    valid = __reduce_add_sync(0xffffffffu, valid);  // blocks are whole warps
-    if ((threadIdx.x & 31) == 0 && valid) atomicAdd(&st->total, valid);
-    __syncthreads();
-    for (int j = threadIdx.x; j < kSlots; j += blockDim.x)
-        if (slot_cnt[j]) atomicAdd(&hist[slot_bin[j]], slot_cnt[j]);
-}
-
-// Histogram of the next 16 bits among keys that match the selected prefix.
-__global__ void k_sel_hist(const unsigned long long *__restrict__ keys, int64_t P, int pass,
-                           unsigned int *__restrict__ hist, const SelState *st) {
-    const int hi_shift = 64 - 16 * pass;  // bits above this are fixed
-    const unsigned long long prefix = st->prefix;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < P; i += (int64_t)gridDim.x * blockDim.x) {
-        const unsigned long long key = keys[i];
-        if (key != 0ull && (key >> hi_shift) == (prefix >> hi_shift))
-            atomicAdd(&hist[(key >> (hi_shift - 16)) & 0xFFFFull], 1u);
-    }
-}
-
-// One CTA: find, from the top, the bin holding the `need`-th largest key,
-// extend the prefix, and clear the histogram.  Thread t sums the 64 bins
-// 65535 - 64 t .. 65472 - 64 t; a block scan of those sums gives each thread
-// the count above its bins, and the one thread whose range holds the
-// need-th key walks its 64 bins.
-__global__ void __launch_bounds__(1024) k_sel_pick(unsigned int *__restrict__ hist, int pass, SelState *st,
-                                                   unsigned int k_top) {
-    __shared__ unsigned int warp_sum[32];
-    __shared__ unsigned int chosen_bin, above;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    if (pass == 0) {
-        if (tid == 0) {
-            st->need = st->total < k_top ? st->total : k_top;
-            st->prefix = 0ull;
-        }
-        __syncthreads();
-    }
-    const unsigned int need = st->need;
-    unsigned int sum = 0;
-    for (int j = 0; j < 64; j++) sum += hist[65535 - (tid * 64 + j)];
-    // inclusive scan over the block, thread order = bins from the top
-    unsigned int inc = sum;
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-        const unsigned int o = __shfl_up_sync(0xffffffffu, inc, d);
-        if (lane >= d) inc += o;
-    }
-    if (lane == 31) warp_sum[warp] = inc;
-    if (tid == 0) {
-        chosen_bin = 0;
-        above = 0;
-    }
-    __syncthreads();
-    if (warp == 0) {
-        const unsigned int w = warp_sum[lane];
-        unsigned int wi = w;
-#pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            const unsigned int o = __shfl_up_sync(0xffffffffu, wi, d);
-            if (lane >= d) wi += o;
-        }
-        warp_sum[lane] = wi - w;  // keys in the bins of earlier warps
-    }
-    __syncthreads();
-    const unsigned int before = warp_sum[warp] + inc - sum;  // keys in bins above this thread's
-    if (need > 0 && before < need && before + sum >= need) {
-        unsigned int acc = before;
-        for (int j = 0; j < 64; j++) {
-            const unsigned int b = 65535 - (tid * 64 + j);
-            if (acc + hist[b] >= need) {
-                chosen_bin = b;
-                above = acc;
-                break;
-            }
-            acc += hist[b];
-        }
-    }
-    __syncthreads();
-    for (int j = tid; j < 65536; j += blockDim.x) hist[j] = 0u;
-    if (tid == 0) {
-        const int shift = 48 - 16 * pass;
-        st->prefix |= (unsigned long long)chosen_bin << shift;
-        st->need = need - above;
-        if (pass == 3) st->thresh = need == 0 ? ~0ull : st->prefix;
-    }
-}
-
-__global__ void k_sel_compact(const unsigned long long *__restrict__ keys, int64_t P,
-                              unsigned long long *__restrict__ out, SelState *st, unsigned int cap) {
-    const unsigned long long th = st->thresh;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < P; i += (int64_t)gridDim.x * blockDim.x) {
-        const unsigned long long key = keys[i];
-        if (key != 0ull && key >= th) {
-            const unsigned int slot = atomicAdd(&st->count, 1u);
-            if (slot < cap) out[slot] = key;
-        }
-    }
-}
-
-// One CTA bitonic sort (descending) of up to kMaxTop keys in shared memory.
-__global__ void __launch_bounds__(1024) k_sel_sort(unsigned long long *__restrict__ keys, const SelState *st,
-                                                   unsigned int cap) {
-    extern __shared__ unsigned long long sk[];
-    unsigned int n = st->count < cap ? st->count : cap;
-    unsigned int m = 1;
-    while (m < n) m <<= 1;
-    for (unsigned int i = threadIdx.x; i < m; i += blockDim.x) sk[i] = i < n ? keys[i] : 0ull;
-    __syncthreads();
-    for (unsigned int size = 2; size <= m; size <<= 1) {
-        for (unsigned int stride = size >> 1; stride > 0; stride >>= 1) {
-            for (unsigned int i = threadIdx.x; i < m; i += blockDim.x) {
-                const unsigned int j = i ^ stride;
-                if (j > i) {
-                    const bool desc = (i & size) == 0;
-                    const unsigned long long a = sk[i], b = sk[j];
-                    if (desc ? (a < b) : (a > b)) {
-                        sk[i] = b;
-                        sk[j] = a;
-                    }
-                }
-            }
-            __syncthreads();
-        }
-    }
-    for (unsigned int i = threadIdx.x; i < n; i += blockDim.x) keys[i] = sk[i];
-}
-
-template <typename TIn>
-__device__ __forceinline__ double to_f64(TIn v) { return (double)to_f32(v); }
-
-// One warp per candidate: N and D in FP64 from the master stack, the FP64
-// footprints and the FP64 inverse variance.
 // FP64 inverse variance of every pixel for the re-score: 1 / (s * s) from
 // the FP32 noise value s in FP64, 0 where the pixel is masked or s is not a
 // usable noise value (s <= 0 or not finite; a finite FP32 s never makes the
@@ -1574,132 +1401,132 @@ __global__ void k_lambda64(const float *__restrict__ sigma, const uint8_t *__res
     }
 }
 
+// One candidate per `wpc` warps (1, 2, 4 or 8: a block holds whole
+// candidates), each taking a share of the frames.
+//
+// N: lanes 0 .. 24 are the footprint's taps; per frame a warp reads the 25
+// FP64 taps (200 consecutive bytes) and the five rows of five stack values,
+// and adds w (s r) into a sum per tap; the sums meet lambda only when the
+// trajectory's base pixel changes (a slow mover stays on a pixel for tens of
+// frames), so a frame costs one FP64 FMA.  D: lambda does not depend on the
+// frame, so D is the collapsed kernel G_k (FP64, a few hundred taps) against
+// lambda, half a warp per run of it.
+//
+// Bound: the FP64 pipe (one warp instruction per 64 cycles and scheduler) and
+// the scattered reads.  The form with lanes over frames -- 25 taps of four FP64 operations and a
+// conversion each, for N and D, and 75 scattered reads per 32 frames --
+// measured 1490 us for 4096 candidates of 1000 frames of 1024^2; this one 530
+// (FP64 pipe 45 %, 2.3 GB of scattered 64-byte DRAM reads in that time).
+// Four frames in flight and 32 warps per SM, so that 4096 candidates run at
+// once; eight frames and 16 warps: 640 us.
 template <typename TIn>
-__global__ void k_rescore(const TIn *__restrict__ r, int64_t fstride, int64_t rstride,
-                          const float *__restrict__ scale, const double *__restrict__ lam64,
-                          const double *__restrict__ taps64,
-                          const int32_t *__restrict__ shifts, const float *__restrict__ snr_max,
-                          const int32_t *__restrict__ argmax, const unsigned long long *__restrict__ keys,
-                          const SelState *st, unsigned int cap, int T, int64_t H, int64_t W,
-                          mf_candidate *__restrict__ out, int32_t *__restrict__ n_out) {
-    const unsigned int n = st->count < cap ? st->count : cap;
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (warp == 0 && lane == 0) *n_out = (int32_t)n;
-    if ((unsigned)warp >= n) return;
-    const unsigned long long key = keys[warp];
-    const int64_t idx = (int64_t)(0xFFFFFFFFu - (uint32_t)(key & 0xFFFFFFFFull));
-    const int64_t py = idx / W, px = idx % W;
-    const int k = argmax[idx];
+__global__ void __launch_bounds__(256, 4) k_rescore(
+    const TIn *__restrict__ r, int64_t fstride, int64_t rstride, const float *__restrict__ scale,
+    const double *__restrict__ lam64, const double *__restrict__ taps64, const int2 *__restrict__ shifts,
+    const RunRec *__restrict__ runs, const int32_t *__restrict__ run_off, const double *__restrict__ wts64,
+    const float *__restrict__ snr_max, const int32_t *__restrict__ argmax,
+    const unsigned long long *__restrict__ keys, const SelState *st, int wpc, int T, int64_t H, int64_t W,
+    mf_candidate *__restrict__ out, int32_t *__restrict__ n_out) {
+    constexpr int U = 4;  // frames whose loads are in flight together
+    __shared__ double part_n[8], part_d[8];
+    const unsigned int n = st->count;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const unsigned int cand = (blockIdx.x * 8u + warp) / (unsigned)wpc;
+    const int part = warp % wpc;
+    if (blockIdx.x == 0 && threadIdx.x == 0) *n_out = (int32_t)n;
+    const bool on = cand < n;
     double num = 0.0, den = 0.0;
-    for (int t = lane; t < T; t += 32) {
-        const size_t kt = (size_t)k * T + t;
-        const int sx = shifts[kt * 2 + 0], sy = shifts[kt * 2 + 1];
-        const double sc = scale ? (double)scale[t] : 1.0;
-        const double *w = taps64 + kt * 25;
-        for (int b = 0; b < 5; b++) {
-            const int64_t qy = py + sy + b - 2;
-            if (qy < 0 || qy >= H) continue;
-            for (int a = 0; a < 5; a++) {
-                const int64_t qx = px + sx + a - 2;
-                if (qx < 0 || qx >= W) continue;
-                const int64_t q = qy * W + qx;
-                const double lam = lam64[q];
-                if (lam == 0.0) continue;  // masked, or no usable noise value
-                const double wl = w[b * 5 + a] * lam;  // w lambda, shared by both sums
-                num = fma(wl, sc * to_f64(r[t * fstride + qy * rstride + qx]), num);
-                den = fma(w[b * 5 + a], wl, den);
+    int64_t idx = 0;
+    int k = 0;
+    if (on) {
+        idx = (int64_t)(0xFFFFFFFFu - (uint32_t)(keys[cand] & 0xFFFFFFFFull));
+        k = argmax[idx];
+        const int Hi = (int)H, Wi = (int)W;  // at most 2^20
+        const int py = (int)(idx / W), px = (int)(idx % W);
+        const int b = lane / 5 - 2, a = lane % 5 - 2;
+        const int t0 = (int)((int64_t)T * part / wpc), t1 = (int)((int64_t)T * (part + 1) / wpc);
+        const size_t kt = (size_t)k * T;
+        int2 base = make_int2(INT_MIN, INT_MIN);
+        double lam = 0.0, acc = 0.0;
+        const TIn *src = r;
+        bool use = false;
+        for (int t = t0; t < t1; t += U) {
+            int2 s[U];
+            double w[U];
+            float v[U];
+#pragma unroll
+            for (int u = 0; u < U; u++) {
+                const int q = min(t + u, t1 - 1);
+                s[u] = shifts[kt + q];
+                w[u] = lane < 25 && t + u < t1 ? taps64[(kt + q) * 25 + lane] : 0.0;
+            }
+#pragma unroll
+            for (int u = 0; u < U; u++) {
+                const int qy = py + s[u].y + b, qx = px + s[u].x + a;
+                const bool in = lane < 25 && t + u < t1 && (unsigned)qy < (unsigned)Hi && (unsigned)qx < (unsigned)Wi;
+                v[u] = in ? to_f32(src[(t + u) * fstride + qy * rstride + qx]) : 0.f;
+            }
+#pragma unroll
+            for (int u = 0; u < U; u++) {
+                if (s[u].x != base.x || s[u].y != base.y) {  // the same for the whole warp
+                    num = fma(lam, acc, num);
+                    acc = 0.0;
+                    base = s[u];
+                    const int qy = py + base.y + b, qx = px + base.x + a;
+                    const bool in = lane < 25 && (unsigned)qy < (unsigned)Hi && (unsigned)qx < (unsigned)Wi;
+                    lam = in ? lam64[qy * W + qx] : 0.0;
+                    use = (__double2hiint(lam) | __double2loint(lam)) != 0;  // else masked, or no usable noise value: the stack's value does not matter
+                }
+                const double x = widen(use ? v[u] : 0.f);
+                if (scale) acc = fma(w[u], (double)scale[min(t + u, t1 - 1)] * x, acc);
+                else acc = fma(w[u], x, acc);
             }
         }
-    }
+        num = fma(lam, acc, num);
+        // D: run r of G_k by half warps
+        const int r1 = run_off[k + 1];
+        for (int q = run_off[k] + 2 * part + (lane >> 4); q < r1; q += 2 * wpc) {
+            const RunRec rr = runs[q];
+            const int y = py + rr.dy;
+            if ((unsigned)y >= (unsigned)Hi) continue;
+            for (int c = lane & 15; c < 4 * rr.nch; c += 16) {
+                const int x = px + rr.x0 + c;
+                if ((unsigned)x < (unsigned)Wi) den = fma(wts64[rr.woff + c], lam64[y * W + x], den);
+            }
+        }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        num += __shfl_xor_sync(0xffffffffu, num, o);
-        den += __shfl_xor_sync(0xffffffffu, den, o);
+        for (int o = 16; o > 0; o >>= 1) {
+            num += __shfl_xor_sync(0xffffffffu, num, o);
+            den += __shfl_xor_sync(0xffffffffu, den, o);
+        }
     }
-    if (lane == 0) {
+    if (wpc > 1) {
+        if (lane == 0) {
+            part_n[warp] = num;
+            part_d[warp] = den;
+        }
+        __syncthreads();
+        if (part != 0) return;
+        for (int w = 1; w < wpc; w++) {
+            num += part_n[warp + w];
+            den += part_d[warp + w];
+        }
+    }
+    if (on && lane == 0) {
         mf_candidate c;
-        c.y = (int32_t)py;
-        c.x = (int32_t)px;
+        c.y = (int32_t)(idx / W);
+        c.x = (int32_t)(idx % W);
         c.k = k;
         c.reserved = 0;
         c.snr = den > 0.0 ? num / sqrt(den) : 0.0;
         c.flux = den > 0.0 ? num / den : 0.0;
         c.snr_search = snr_max[idx];
         c.reserved2 = 0.f;
-        out[warp] = c;
+        out[cand] = c;
     }
 }
 
 }  // namespace
-
-SelectLayout select_layout(int64_t P, int32_t k_top) {
-    SelectLayout L;
-    size_t off = 0;
-    auto take = [&](size_t bytes) {
-        const size_t o = off;
-        off = (off + bytes + 255) / 256 * 256;
-        return o;
-    };
-    L.keys_off = take((size_t)P * sizeof(unsigned long long));
-    L.hist_off = take(65536 * sizeof(unsigned int));
-    L.st_off = take(sizeof(SelState));
-    L.top_off = take((size_t)k_top * sizeof(unsigned long long));
-    L.total = off;
-    return L;
-}
-
-int launch_select(const float *score, const int32_t *valid, int64_t P, int32_t k_top, char *ws,
-                  const SelectLayout &L, void *stream_, char *err, size_t errlen) {
-    cudaStream_t stream = (cudaStream_t)stream_;
-    if (k_top > kMaxTop) {
-        snprintf(err, errlen, "k_top above %d", kMaxTop);
-        return (int)cudaErrorInvalidValue;
-    }
-    unsigned long long *keys = reinterpret_cast<unsigned long long *>(ws + L.keys_off);
-    unsigned int *hist = reinterpret_cast<unsigned int *>(ws + L.hist_off);
-    SelState *sst = reinterpret_cast<SelState *>(ws + L.st_off);
-    unsigned long long *top = reinterpret_cast<unsigned long long *>(ws + L.top_off);
-    cudaError_t e = cudaMemsetAsync(ws + L.hist_off, 0, L.top_off - L.hist_off, stream);
-    if (e != cudaSuccess) {
-        snprintf(err, errlen, "cudaMemsetAsync: %s", cudaGetErrorString(e));
-        return (int)e;
-    }
-    {
-        LaunchScope ls(kKSelect, stream);
-        k_sel_keys<<<grid_for(P, 256), 256, 0, stream>>>(score, valid, P, keys, hist, sst);
-    }
-    MF_CHECK_LAUNCH("k_sel_keys");
-    for (int pass = 0; pass < 4; pass++) {
-        if (pass > 0) {
-            LaunchScope ls(kKSelect, stream);
-            k_sel_hist<<<grid_for(P, 256), 256, 0, stream>>>(keys, P, pass, hist, sst);
-            MF_CHECK_LAUNCH("k_sel_hist");
-        }
-        LaunchScope ls(kKSelect, stream);
-        k_sel_pick<<<1, 1024, 0, stream>>>(hist, pass, sst, (unsigned)k_top);
-        MF_CHECK_LAUNCH("k_sel_pick");
-    }
-    {
-        LaunchScope ls(kKCompact, stream);
-        k_sel_compact<<<grid_for(P, 256), 256, 0, stream>>>(keys, P, top, sst, (unsigned)k_top);
-    }
-    MF_CHECK_LAUNCH("k_sel_compact");
-    {
-        unsigned int m = 1;
-        while (m < (unsigned)k_top) m <<= 1;
-        const size_t smem = (size_t)m * sizeof(unsigned long long);
-        e = cudaFuncSetAttribute(k_sel_sort, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) {
-            snprintf(err, errlen, "cudaFuncSetAttribute(sort): %s", cudaGetErrorString(e));
-            return (int)e;
-        }
-        LaunchScope ls(kKSort, stream);
-        k_sel_sort<<<1, 1024, smem, stream>>>(top, sst, (unsigned)k_top);
-    }
-    MF_CHECK_LAUNCH("k_sel_sort");
-    return 0;
-}
 
 size_t rescore_workspace(int64_t H, int64_t W, int32_t k_top) { return select_layout(H * W, k_top).total; }
 
@@ -1724,27 +1551,21 @@ int launch_rescore(const RescoreArgs &a, char *err, size_t errlen) {
     }
     MF_CHECK_LAUNCH("k_lambda64");
     {
-        const int threads = 256;
-        const int blocks = (int)(((int64_t)a.k_top * 32 + threads - 1) / threads);
+        // enough warps to fill the chip (24 per SM) when candidates are few
+        int wpc = 1;
+        while (wpc < 8 && (int64_t)a.k_top * wpc < 152 * 24) wpc *= 2;
+        const unsigned blocks = (unsigned)(((int64_t)a.k_top * wpc + 7) / 8);
         LaunchScope ls(kKRescore, stream);
-        const int64_t fs = st.frame_stride, rs = st.row_stride;
-        switch (st.dtype) {
-            case MF_F32:
-                k_rescore<float><<<blocks, threads, 0, stream>>>(
-                    (const float *)st.data, fs, rs, st.frame_scale, lam64, tab.d_taps64, tab.d_shifts,
-                    a.snr_max, a.argmax, top, sst, (unsigned)a.k_top, tab.T, H, W, a.out, a.n_out);
-                break;
-            case MF_BF16:
-                k_rescore<__nv_bfloat16><<<blocks, threads, 0, stream>>>(
-                    (const __nv_bfloat16 *)st.data, fs, rs, st.frame_scale, lam64, tab.d_taps64,
-                    tab.d_shifts, a.snr_max, a.argmax, top, sst, (unsigned)a.k_top, tab.T, H, W, a.out, a.n_out);
-                break;
-            default:
-                k_rescore<__half><<<blocks, threads, 0, stream>>>(
-                    (const __half *)st.data, fs, rs, st.frame_scale, lam64, tab.d_taps64, tab.d_shifts,
-                    a.snr_max, a.argmax, top, sst, (unsigned)a.k_top, tab.T, H, W, a.out, a.n_out);
-                break;
-        }
+        auto go = [&](auto t) {
+            using TI = decltype(t);
+            k_rescore<TI><<<blocks, 256, 0, stream>>>(
+                (const TI *)st.data, st.frame_stride, st.row_stride, st.frame_scale, lam64, tab.d_taps64,
+                reinterpret_cast<const int2 *>(tab.d_shifts), tab.d_runs, tab.d_run_off, tab.d_wts64, a.snr_max,
+                a.argmax, top, sst, wpc, tab.T, H, W, a.out, a.n_out);
+        };
+        if (st.dtype == MF_F32) go(float{});
+        else if (st.dtype == MF_BF16) go(__nv_bfloat16{});
+        else go(__half{});
     }
     MF_CHECK_LAUNCH("k_rescore");
     return 0;

@@ -189,3 +189,24 @@ def test_detect_full_size_paper_shaped(mf, oracle):
     s, a = synth.score_map(2048, 2048, seed=3, K=100)
     checked, found = _compare(mf, oracle, s, a, 255, 3.0)
     assert found > 1000 and checked > 0.95 * found
+
+
+@pytest.mark.parametrize("H,W,window,threshold,submean", [
+    (9, 2049, 31, 2.5, True),      # one column past a row tile
+    (40, 2080, 63, -5.0, True),    # nearly every pixel a candidate, one huge component
+    (130, 190, 3, 0.9, True),      # more detections than are ranked at once
+    (57, 33, 2047, 2.0, False),
+])
+def test_detect_tiles_and_crowds(mf, oracle, H, W, window, threshold, submean):
+    from paper_2209_09848_gb300 import synth
+    s, a = synth.score_map(H, W, seed=H + W, K=7, n_sources=40)
+    _compare(mf, oracle, s, a, window, threshold, submean, max_out=300)
+
+
+@pytest.mark.parametrize("scale", [1e-30, 1e-12, 1e25])
+def test_detect_far_scales(mf, oracle, scale):
+    # z does not depend on the scale of the scores; at these the FP32 form of
+    # z would leave its range and the FP64 formula takes over
+    from paper_2209_09848_gb300 import synth
+    s, a = synth.score_map(90, 333, seed=5, K=7)
+    _compare(mf, oracle, s * np.float32(scale), a, 15, 3.0)

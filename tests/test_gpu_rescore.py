@@ -93,3 +93,53 @@ def test_rescore_argument_errors(mf):
         mf.rescore_topk(r, s, table, smax, amax, 0)
     with pytest.raises(mf.MFError):
         mf.rescore_topk(r, s, table, smax, amax, H * W + 1)
+
+
+@pytest.mark.parametrize("kind", ["noise", "constant", "rounded", "negative", "wide", "infinite"])
+@pytest.mark.parametrize("valid", [1.0, 0.001])
+def test_selection_of_hard_maps(mf, oracle, kind, valid):
+    # ties by the hundred thousand (the list past the ranking's limit is cut
+    # by the radix select), every sign and exponent, few valid pixels; the
+    # selection is exact integer work
+    H, W = 371, 523
+    g = np.random.default_rng(len(kind))
+    m = {"noise": lambda: g.normal(2.5, 0.45, (H, W)), "constant": lambda: np.full((H, W), 2.5),
+         "rounded": lambda: np.round(g.normal(2.5, 0.45, (H, W)), 1), "negative": lambda: -np.abs(g.normal(size=(H, W))),
+         "wide": lambda: g.normal(size=(H, W)) * 10.0 ** g.uniform(-40, 30, (H, W)),
+         "infinite": lambda: np.where(g.random((H, W)) < 0.1, np.inf, g.normal(size=(H, W)))}[kind]().astype(np.float32)
+    a = np.where(g.random((H, W)) < valid, 0, -1).astype(np.int32)
+    table = mf.prf_table_create([0.0], [0.0], 1)
+    r, sg = torch.zeros((1, H, W), device="cuda"), torch.ones((H, W), device="cuda")
+    for k in (1, 33, 4096, 16384):
+        raw, n = mf.rescore_topk(r, sg, table, torch.from_numpy(m).cuda(), torch.from_numpy(a).cuda(), k)
+        c = mf.decode_candidates(raw, int(n.item()))
+        assert np.array_equal(c["y"].astype(np.int64) * W + c["x"], oracle.topk_order(m, a, k))
+
+
+@pytest.mark.parametrize("k_top,T", [(3, 37), (700, 9), (2500, 5)])
+def test_rescore_custom_footprints_and_scales(mf, oracle, k_top, T):
+    # candidates shared by 8, 8 and 2 warps; a base pixel that changes every
+    # frame, footprints that do not factor, frame scales, and a masked pixel
+    # holding NaN (its value does not matter); 1e-9: FP64 sums in other orders
+    from paper_2209_09848_gb300 import synth
+    H, W, K = 61, 70, 5
+    c = synth.small_case(T, H, W, 40 + T, mask_frac=0.03, movers=1)
+    g = np.random.default_rng(T)
+    sh = g.integers(-9, 10, size=(K, T, 2)).astype(np.int32)
+    tp = g.uniform(-0.2, 1.0, size=(K, T, 5, 5))
+    table = mf.prf_table_create_custom(sh, tp)
+    scale = g.uniform(0.5, 2.0, T).astype(np.float32)
+    res = np.where(c["mask"][None] > 0, np.nan, c["res"]).astype(np.float32)
+    s_max, a_max = synth.score_map(H, W, seed=T, K=K, mask_frac=0.0)
+    dev = "cuda"
+    raw, n = mf.rescore_topk(torch.from_numpy(res).to(dev), torch.from_numpy(c["sigma"]).to(dev), table,
+                             torch.from_numpy(s_max).to(dev), torch.from_numpy(a_max).to(dev), k_top,
+                             mask=torch.from_numpy(c["mask"]).to(dev), frame_scale=torch.from_numpy(scale).to(dev))
+    got = mf.decode_candidates(raw, int(n.item()))
+    want = oracle.topk_order(s_max, a_max, k_top)
+    lam = oracle.inverse_variance(c["sigma"], c["mask"])
+    N, D = oracle.search_points(c["res"], lam, sh, tp, (want // W).astype(np.int32), (want % W).astype(np.int32),
+                                a_max.ravel()[want], frame_scale=scale.astype(np.float64))
+    ok = D > 0
+    np.testing.assert_allclose(got["snr"][ok], N[ok] / np.sqrt(D[ok]), rtol=1e-9, atol=1e-9)
+    np.testing.assert_allclose(got["flux"][ok], N[ok] / D[ok], rtol=1e-9, atol=1e-9)
