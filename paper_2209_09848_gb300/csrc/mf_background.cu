@@ -493,7 +493,7 @@ int launch_refit(const RefitArgs &a, char *err, size_t errlen) {
         const Resident r = pick_resident(a.T, vec);
         const int groups = 32 * r.nw / r.quads, np = (int)((a.T + 2 * groups - 1) / (2 * groups));
         const size_t smem = (size_t)np * (2 * 32 * r.nw + 3 * groups) * sizeof(float4);
-        e = cudaFuncSetAttribute(r.kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        e = cudaFuncSetAttribute(r.kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemAllowStatic);
         if (e == cudaSuccess) {
             const int64_t nblk = (P + 4 * r.quads - 1) / (4 * r.quads), ctas = (int64_t)152 * (kResWarps / r.nw);
             const ProfToken tok = prof_begin(kKRefit, stream);

@@ -539,7 +539,7 @@ int launch_detect(const DetectArgs &a, char *err, size_t errlen) {
     {
         const int tile = std::min(kRowTile, (W + 31) / 32 * 32);
         const size_t smem = (size_t)(tile + 2 * R + 1) * (8 + 8 + 4);
-        e = cudaFuncSetAttribute(k_det_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        e = cudaFuncSetAttribute(k_det_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemAllowStatic);
         if (e != cudaSuccess) {
             snprintf(err, errlen, "cudaFuncSetAttribute(k_det_rows): %s", cudaGetErrorString(e));
             return (int)e;

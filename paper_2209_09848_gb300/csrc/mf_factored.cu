@@ -11,11 +11,14 @@
 // general 5 x 5 stencil; the arithmetic is the same sum regrouped.
 //
 // Per pair of frames (t, t + 1): every thread waits for both windows (TMA
-// boxes, mbarriers with bounded waits); the CTA's threads split both row
-// passes into items of 16 outputs (the column phase is applied as an item
-// reads the window, so the row-pass buffer holds exactly the tile's columns;
-// items go to the last warps first, so the row-pass-only warps that round a
-// CTA up to a multiple of 4 warps and the warps of empty slots take them);
+// boxes, mbarriers with bounded waits); the CTA's warps split both row passes
+// into units of 32 rows x 16 columns, an item of 16 outputs per lane (the
+// column phase is applied as an item reads the window, so the row-pass buffer
+// holds exactly the tile's columns; units go to the last warps first, so the
+// row-pass-only warps that round a CTA up to a multiple of 4 warps and the
+// warps of empty slots take them; a unit's frame, phase and addresses are
+// uniform over its warp: 2.7 % faster than items dealt to threads, whatever
+// their frame);
 // one CTA barrier; thread 0 refills both
 // stages with frames t + stages and t + 1 + stages; each warp runs the
 // column passes of its (trajectory slot, 32 x 32 sub-tile) for both frames:
@@ -178,7 +181,9 @@ __device__ __forceinline__ bool fac_tile(const CUtensorMap &ymap, const FacParam
         }
         if (!any) return true;  // same for every thread of the CTA
     }
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    // from lane 0, so that the compiler knows the warp's index to be uniform
+    const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
+    const int nwarps = blockDim.x >> 5;
     const int nsub = (p.th / 32) * NSUBX;
     // a slot's warps are consecutive, so they spread over the SM's four
     // schedulers and an empty slot leaves every scheduler the same work
@@ -246,26 +251,27 @@ __device__ __forceinline__ bool fac_tile(const CUtensorMap &ymap, const FacParam
         acc[r] = 0.f;
         blk[r] = 0.f;
     }
-    auto record = [&](int f) { return fb + (((f / R) & 1) * R + f % R) * kBB; };
-    auto column = [&](int f) {
-        if (!active) return;
-        const unsigned char *fblk = record(f);
-        const FacSlot *fs = reinterpret_cast<const FacSlot *>(fblk + sizeof(FacHdr)) + slot;
+    static_assert(2 * R == 16, "a frame's record stands at its index mod 16");
+    auto record = [&](int f) { return fb + (f & 15) * kBB; };
+    // the column pass of one frame: its records at rec, its row-pass buffer at h
+    const int lane_off = (32 * sub_y + 16 * rh) * HP + 32 * sub_x + 2 * cp;
+    auto column = [&](const unsigned char *rec, const float *h) {
+        const FacSlot *fs = reinterpret_cast<const FacSlot *>(rec + sizeof(FacHdr)) + slot;
         const float4 u4 = *reinterpret_cast<const float4 *>(fs->uy);
         const float2 u5 = *reinterpret_cast<const float2 *>(fs->uy + 4);  // u_y(2) and the row offset
         const float u[5] = {u4.x, u4.y, u4.z, u4.w, u5.x};
-        const float *col = hbuf + (size_t)(f % kFacHBufs) * BH * HP + (32 * sub_y + 16 * rh + __float_as_int(u5.y)) * HP + 32 * sub_x + 2 * cp;
+        const float *col = h + lane_off + __float_as_int(u5.y) * HP;
         // taps b = B0 .. B1 of the footprint (all five, or the centre one)
         constexpr int B0 = 2 - TAPS / 2, B1 = 2 + TAPS / 2;
 #pragma unroll
         for (int i = B0; i < 16 + B1; i++) {
-            const float2 h = *reinterpret_cast<const float2 *>(col + i * HP);
+            const float2 hv = *reinterpret_cast<const float2 *>(col + i * HP);
 #pragma unroll
             for (int b = B0; b <= B1; b++) {
                 const int r = i - b;
                 if (r >= 0 && r < 16) {
-                    blk[2 * r] = fmaf(u[b], h.x, blk[2 * r]);
-                    blk[2 * r + 1] = fmaf(u[b], h.y, blk[2 * r + 1]);
+                    blk[2 * r] = fmaf(u[b], hv.x, blk[2 * r]);
+                    blk[2 * r + 1] = fmaf(u[b], hv.y, blk[2 * r + 1]);
                 }
             }
         }
@@ -291,27 +297,29 @@ __device__ __forceinline__ bool fac_tile(const CUtensorMap &ymap, const FacParam
             for (int r = 0; r < 32; r++) blk[r] += Win<E>::one(col + r * RP);
         }
     };
-    // the row passes of frames f0 (stage s0) and f0 + 1 (stage s1, if it
-    // exists) as one list of items: item it < n0 is (row, m) of frame f0
-    auto row_pair = [&](int f0, int s0, int s1, bool two) {
-        const FacHdr *h0 = reinterpret_cast<const FacHdr *>(record(f0));
-        const FacHdr *h1 = reinterpret_cast<const FacHdr *>(record(two ? f0 + 1 : f0));
-        const int n0 = h0->nrows * NI, n1 = two ? h1->nrows * NI : 0;
-        for (int it = (int)blockDim.x - 1 - (int)threadIdx.x; it < n0 + n1; it += blockDim.x) {
+    // the row passes of frames f0 (records rec0, window w0, buffer h0) and f0 +
+    // 1 (if `two`; records, window w1, buffer h1 likewise), in units of 32 rows
+    // x 16 columns, an item per lane: a unit has one frame, one column phase
+    // and one address stride, so its set-up is uniform over the warp
+    auto row_pair = [&](int f0, const unsigned char *rec0, const E *w0, const E *w1, float *h0, float *h1, bool two) {
+        const unsigned char *rec1 = rec0 + (two ? kBB : 0u);
+        const int rows0 = reinterpret_cast<const FacHdr *>(rec0)->nrows - p.dth;
+        const int rows1 = two ? reinterpret_cast<const FacHdr *>(rec1)->nrows - p.dth : 0;
+        const int n0 = ((rows0 + 31) >> 5) * NI, n1 = ((rows1 + 31) >> 5) * NI;
+        for (int it = nwarps - 1 - warp; it < n0 + n1; it += nwarps) {
             const bool second = it >= n0;
-            const FacHdr *fh = second ? h1 : h0;
-            const int f = second ? f0 + 1 : f0, st = second ? s1 : s0, j = second ? it - n0 : it;
-            const int nrows = fh->nrows;
-            const int m = (int)(((float)j + 0.5f) * fh->inv_nrows), row = j - m * nrows;
-            const E *src = rwin + (size_t)st * SF * EPF + row * RP + kFacItem * m;
-            float *dst = hbuf + (size_t)(QG ? (f & 1) : f % kFacHBufs) * BH * HP + row * HP + kFacItem * m;
+            const int j = second ? it - n0 : it, m = j % NI, row = (j / NI) * 32 + lane;
+            const float4 *hd = reinterpret_cast<const float4 *>(second ? rec1 : rec0);
+            const float4 ua = hd[1], ub = hd[2];  // u_x(-2 .. 1); u_x(2), 1 / nrows, column phase of 16-bit windows
+            if (row >= (second ? rows1 : rows0)) continue;
+            const E *src = (second ? w1 : w0) + row * RP + kFacItem * m;
+            float *dst = (second ? h1 : h0) + row * HP + kFacItem * m;
             if constexpr (k16) {
                 // the taps carry the frame's scale of a 16-bit weighted stack
                 // (a power of two: u_x * beta is exact)
-                const float bt = p.beta ? p.beta[f] : 1.f;
-                const float ux0 = fh->ux[0] * bt, ux1 = fh->ux[1] * bt, ux2 = fh->ux[2] * bt,
-                            ux3 = fh->ux[3] * bt, ux4 = fh->ux[4] * bt;
-                switch (fh->cofs8) {
+                const float bt = p.beta ? p.beta[second ? f0 + 1 : f0] : 1.f;
+                const float ux0 = ua.x * bt, ux1 = ua.y * bt, ux2 = ua.z * bt, ux3 = ua.w * bt, ux4 = ub.x * bt;
+                switch (__float_as_int(ub.z)) {
                     case 0: row_item<0, TAPS>(src, dst, ux0, ux1, ux2, ux3, ux4); break;
                     case 1: row_item<1, TAPS>(src, dst, ux0, ux1, ux2, ux3, ux4); break;
                     case 2: row_item<2, TAPS>(src, dst, ux0, ux1, ux2, ux3, ux4); break;
@@ -322,12 +330,11 @@ __device__ __forceinline__ bool fac_tile(const CUtensorMap &ymap, const FacParam
                     default: row_item<7, TAPS>(src, dst, ux0, ux1, ux2, ux3, ux4); break;
                 }
             } else {
-                const float ux0 = fh->ux[0], ux1 = fh->ux[1], ux2 = fh->ux[2], ux3 = fh->ux[3], ux4 = fh->ux[4];
-                switch (fh->cofs) {
-                    case 0: row_item<0, TAPS>(src, dst, ux0, ux1, ux2, ux3, ux4); break;
-                    case 1: row_item<1, TAPS>(src, dst, ux0, ux1, ux2, ux3, ux4); break;
-                    case 2: row_item<2, TAPS>(src, dst, ux0, ux1, ux2, ux3, ux4); break;
-                    default: row_item<3, TAPS>(src, dst, ux0, ux1, ux2, ux3, ux4); break;
+                switch (reinterpret_cast<const FacHdr *>(hd)->cofs) {
+                    case 0: row_item<0, TAPS>(src, dst, ua.x, ua.y, ua.z, ua.w, ub.x); break;
+                    case 1: row_item<1, TAPS>(src, dst, ua.x, ua.y, ua.z, ua.w, ub.x); break;
+                    case 2: row_item<2, TAPS>(src, dst, ua.x, ua.y, ua.z, ua.w, ub.x); break;
+                    default: row_item<3, TAPS>(src, dst, ua.x, ua.y, ua.z, ua.w, ub.x); break;
                 }
             }
         }
@@ -412,7 +419,9 @@ __device__ __forceinline__ bool fac_tile(const CUtensorMap &ymap, const FacParam
             const uint32_t par1 = (s + 1 == NS) ? (par ^ 1u) : par;
             bool ready = mbar_wait(smem_u32(&bars[s]), par, 1, p.status);
             if (ready && two) ready = mbar_wait(smem_u32(&bars[s1]), par1, 1, p.status);
-            if (ready) row_pair(t, s, s1, two);
+            if (ready)
+                row_pair(t, record(t), rwin + (size_t)s * SF * EPF, rwin + (size_t)s1 * SF * EPF, hbuf,
+                         hbuf + (size_t)BH * HP, two);
             if (__syncthreads_or(!ready)) {
                 bad = true;
                 break;
@@ -443,12 +452,16 @@ __device__ __forceinline__ bool fac_tile(const CUtensorMap &ymap, const FacParam
             par = (s1 + 1 == NS) ? (par1 ^ 1u) : par1;
         }
     }
-    for (int t = t0; t < t1 && !QG; t += 2) {  // column passes (the loop is empty for QG)
+    int in_block = 0;  // frames in the current partial sums
+    for (int t = t0; t < t1 && !QG; t += 2) {  // column passes (the loop is empty for QG); t is even
         const bool two = t + 1 < t1;
         const int s1 = (s + 1 == NS) ? 0 : s + 1;
         const uint32_t par1 = (s + 1 == NS) ? (par ^ 1u) : par;
         bool ready = mbar_wait(smem_u32(&bars[s]), par, 1, p.status);
         if (ready && two) ready = mbar_wait(smem_u32(&bars[s1]), par1, 1, p.status);
+        const unsigned char *rec = record(t);
+        // row-pass buffers 0, 1 and 2, 3 in turn
+        float *h0 = hbuf + (t & 2) * (BH * HP), *h1 = h0 + BH * HP;
         if (TAPS == 1) {
             // the column passes read the stages themselves: they run before
             // the barrier that frees the stages for refilling
@@ -457,7 +470,7 @@ __device__ __forceinline__ bool fac_tile(const CUtensorMap &ymap, const FacParam
                 if (two) column_direct(t + 1, s1);
             }
         } else if (ready) {
-            row_pair(t, s, s1, two);
+            row_pair(t, rec, rwin + s * (SF * EPF), rwin + s1 * (SF * EPF), h0, h1, two);
         }
         if (__syncthreads_or(!ready)) {
             bad = true;
@@ -467,19 +480,21 @@ __device__ __forceinline__ bool fac_tile(const CUtensorMap &ymap, const FacParam
         if (threadIdx.x == 0) {
             fence_proxy_async();
             if (t + NS < t1) {
-                const FacHdr *fh = reinterpret_cast<const FacHdr *>(record(t));
+                const FacHdr *fh = reinterpret_cast<const FacHdr *>(rec);
                 issue(t + NS, s, fh->next_roy, fh->next_rox);
             }
             if (two && t + 1 + NS < t1) {
-                const FacHdr *fh = reinterpret_cast<const FacHdr *>(record(t + 1));
+                const FacHdr *fh = reinterpret_cast<const FacHdr *>(rec + kBB);
                 issue(t + 1 + NS, s1, fh->next_roy, fh->next_rox);
             }
         }
-        if (TAPS != 1) {
-            column(t);
-            if (two) column(t + 1);
+        if (TAPS != 1 && active) {
+            column(rec, h0);
+            if (two) column(rec + kBB, h1);
         }
-        if ((t - t0 + 2) % kFrameBlock == 0) {
+        in_block += 2;
+        if (in_block == kFrameBlock) {
+            in_block = 0;
 #pragma unroll
             for (int r = 0; r < 32; r++) {
                 acc[r] += blk[r];
@@ -601,6 +616,7 @@ __global__ void k_finalize_planes(const float *__restrict__ plane, const float *
             best[v] = 0.f;
             arg[v] = -1;
         }
+#pragma unroll 4
         for (int k = 0; k < K; k++) {
             const VecT xv = reinterpret_cast<const VecT *>(plane + (int64_t)k * P)[i];
             const VecT dv = reinterpret_cast<const VecT *>(isd + (int64_t)k * P)[i];
@@ -632,7 +648,9 @@ int fac_finalize_enqueue(const float *plane, const float *isd, int K, int64_t P,
                          float *snr_all, const int *slot, int *global_status, void *stream, char *err,
                          size_t errlen) {
     if (P <= 0) return 0;
-    const bool vec = P % 4 == 0 && (uintptr_t)snr_all % 16 == 0;
+    // four pixels a thread once they still fill the SMs (128^2 pixels: 64 blocks
+    // of single ones instead of 16)
+    const bool vec = P % 4 == 0 && (uintptr_t)snr_all % 16 == 0 && P >= 4 * 256 * 152;
     const int64_t items = vec ? P / 4 : P;
     int64_t blocks = (items + 255) / 256;
     if (blocks > 152 * 16) blocks = 152 * 16;
@@ -715,7 +733,7 @@ int fac_enqueue(const void *tensor_map, const FacParams &p, int tw, int taps, in
                 long long nblocks, void *stream, char *err, size_t errlen) {
     const CUtensorMap &map = *reinterpret_cast<const CUtensorMap *>(tensor_map);
     FacKernel kern = pick_fac(tw, taps, etype, p.npl > 0);
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemAllow);
     if (e != cudaSuccess) {
         snprintf(err, errlen, "cudaFuncSetAttribute(smem=%zu): %s", smem, cudaGetErrorString(e));
         return (int)e;

@@ -873,13 +873,14 @@ void denominator_layouts(mf_prf_table *t, HostLayouts &out) {
         nr_max = std::max(nr_max, run_off[k + 1] - run_off[k]);
         boxes[k] = b;
     }
+    t->den_rows = rows_max;
+    t->den_cols = cols_max;
+    t->den_nw = nw_max;
+    t->den_nr = nr_max;
     t->den_th = 0;
-    t->den_smem = 0;
     for (int th : {32, 16, 8}) {
-        const size_t sm = mf::den_box_smem(th, rows_max, cols_max, nw_max, nr_max);
-        if (sm <= (size_t)mf::kSmemBudget) {
+        if (mf::den_box_smem(th, rows_max, cols_max, nw_max, nr_max) <= (size_t)mf::kSmemBudget) {
             t->den_th = th;
-            t->den_smem = sm;
             break;
         }
     }
@@ -1009,13 +1010,26 @@ namespace mf {
 
 mf_status set_error(mf_status s, const char *msg) { return fail(s, "%s", msg); }
 
-long long fac_ctas(const mf_prf_table &tab, int64_t H, int64_t W, int seg) {
+long long fac_ctas(const mf_prf_table &tab, int64_t H, int64_t W, int seg, int th) {
     const Plan &p = tab.plan;
     if (seg < 0 || seg >= p.f_seg) return 0;
     const long long tiles_x = (W + p.f_tw - 1) / p.f_tw;
     int spread = 0;
     for (int g = 0; g < p.G; g++) spread = std::max(spread, p.seg_qy[((size_t)g * p.f_seg + seg) * 2 + 1]);
-    return (H + spread + p.f_th - 1) / p.f_th * tiles_x * p.G;
+    return (H + spread + th - 1) / th * tiles_x * p.G;
+}
+
+// A CTA's time is its frames, each at least a barrier and the latencies around
+// it; fewer rows per tile cost more row-pass halo in all but spread a small
+// image over more SMs.  The tallest tile that leaves no SM idle, else 32 rows.
+// 32 frames of 128^2, 16 trajectories: 16 CTAs of 128 rows 39 us, 64 of 32
+// rows 25 us.
+int fac_tile_rows(const mf_prf_table &tab, int64_t H, int64_t W) {
+    const Plan &p = tab.plan;
+    if (p.f_planes > 0) return p.f_th;
+    int th = p.f_th;
+    while (th > 32 && fac_ctas(tab, H, W, 0, th) < 152) th -= 32;
+    return th;
 }
 
 WorkspaceLayout search_layout(int64_t T, int64_t H, int64_t W, int32_t dtype, const mf_prf_table *tab) {

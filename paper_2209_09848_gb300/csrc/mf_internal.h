@@ -32,6 +32,11 @@ constexpr int kDenCols = 256;        // denominator: start pixels per warp (one 
 // registers a thread, which holds the blocked sums of a lane's 32 outputs.
 constexpr int kFacMaxWarps = 20;
 constexpr int kSmemBudget = 220 * 1024;  // dynamic shared memory of one CTA per SM
+// The dynamic shared memory a kernel is allowed (its attribute): one value for
+// every launch, so that threads launching it with different sizes never lower
+// each other's.
+constexpr int kSmemAllow = 224 * 1024;
+constexpr int kSmemAllowStatic = 214 * 1024;  // the same for kernels with static arrays too
 
 // CTA shapes: trajectories per CTA x sub-tiles across x sub-tiles down = kWarps.
 struct Shape {
@@ -76,20 +81,20 @@ struct alignas(16) RunRec {
 
 // Bounding box of G_k's runs: row offsets dy0 .. dy0 + rows - 1, columns x0 ..
 // x0 + cols - 1 (x0 and cols multiples of 4), weights w0 .. w0 + nw - 1.  The
-// staged denominator copies, per (trajectory, tile of th x kDenBoxCols start
-// pixels), the lambda box those start pixels reach into shared memory.
+// staged denominator copies, per (trajectory, tile of th x C start pixels),
+// the lambda box those start pixels reach into shared memory.
 struct alignas(16) DenBox {
     int32_t dy0, rows, x0, cols, w0, nw, pad[2];
 };
-constexpr int kDenBoxCols = 256;  // start pixels per row of a staged-denominator tile
+constexpr int kDenBoxCols = 256;  // start pixels per row of a staged-denominator tile at most
 constexpr int kDenOut = 8;        // start pixels per thread of the staged denominator
 // Row pitch in 16-byte chunks of a staged lambda box for `cols` box columns:
 // odd, so that the same chunk of 8 consecutive rows falls in 8 distinct bank
 // groups.
-__host__ __device__ constexpr int den_pitch(int cols) { return (kDenBoxCols + cols) / 4 | 1; }
+__host__ __device__ constexpr int den_pitch(int cols, int C) { return (C + cols) / 4 | 1; }
 // Box, weights and the trajectory's runs (nruns RunRec) in shared memory.
-inline size_t den_box_smem(int th, int rows, int cols, int nw, int nruns) {
-    return (size_t)(th + rows - 1) * den_pitch(cols) * 16 + (size_t)(nw + 4) * 4 + (size_t)nruns * 16 + 64;
+inline size_t den_box_smem(int th, int rows, int cols, int nw, int nruns, int C = kDenBoxCols) {
+    return (size_t)(th + rows - 1) * den_pitch(cols, C) * 16 + (size_t)(nw + 4) * 4 + (size_t)nruns * 16 + 64;
 }
 
 // ------------------------------------------------ factored numerator ---
@@ -203,7 +208,10 @@ struct Plan {
     int kt() const { return kernel == 2 ? f_kt : kShapes[shape].kt; }
     int tile_h() const { return kernel == 2 ? f_th : kTile * kShapes[shape].tys; }
     int tile_w() const { return kernel == 2 ? f_tw : kTile * kShapes[shape].txs; }
-    int warps() const { return kernel == 2 ? f_kt * (f_th / 32) * (f_tw / 32) : kWarps; }
+    int warps() const { return kernel == 2 ? warps_at(f_th) : kWarps; }
+    // the factored numerator with tiles of th rows (the plan's f_th, or fewer)
+    int warps_at(int th) const { return f_kt * (th / 32) * (f_tw / 32); }
+    size_t smem_at(int th) const;
     // warps launched: the factored kernel rounds up to a multiple of 4 so
     // that each SM scheduler has as many warps; the extra warps make row-pass
     // items only
@@ -218,9 +226,10 @@ inline size_t numerator_smem_bytes(int S, int BH, int kt) {
            (size_t)kStages * sizeof(uint64_t) + 3 * kStages * sizeof(int) + sizeof(int) + 64;
 }
 
-inline size_t Plan::smem() const {
-    return kernel == 2 ? fac_smem_bytes(f_tw, f_bh, f_ns, f_kt, f_planes) : numerator_smem_bytes(S, BH, kt());
+inline size_t Plan::smem_at(int th) const {
+    return fac_smem_bytes(f_tw, f_bh - (f_th - th), f_ns, f_kt, f_planes);
 }
+inline size_t Plan::smem() const { return kernel == 2 ? smem_at(f_th) : numerator_smem_bytes(S, BH, kt()); }
 
 }  // namespace mf
 
@@ -256,7 +265,8 @@ struct mf_prf_table {
     mf::RunRec *d_runs = nullptr;        // [n_seg]
     mf::DenBox *d_boxes = nullptr;       // [K] staged denominator: G_k's bounding box
     int den_th = 0;                      // staged denominator tile rows (0: the unstaged kernel)
-    size_t den_smem = 0;                 // its dynamic shared memory
+    // largest G_k: box rows and columns, weights, runs (the tile's shared memory)
+    int den_rows = 1, den_cols = 4, den_nw = 4, den_nr = 1;
     int32_t *d_run_off = nullptr;        // [K + 1]
     float *d_wts = nullptr;              // run weights
     double *d_wts64 = nullptr;           // the same in FP64 (re-score)
@@ -414,6 +424,7 @@ struct FacParams {
     int *status;                  // the search's status slot
     const float *beta;            // [T] scale of a 16-bit weighted stack, or null (1)
     int T, G, kt, th, bh, ns, S, K;
+    int dth;                      // rows the tile is short of the plan's: so are its windows
     int npl;                      // phase planes per frame block (0: column passes)
     int seg;                      // the segment this launch computes
     int warps;                    // warps of the layout (a batched launch may have more)
@@ -429,7 +440,10 @@ int fac_finalize_enqueue(const float *plane, const float *isd, int K, int64_t P,
                          size_t errlen);
 // CTAs of segment `seg` of a factored search: groups x tile columns x tile
 // rows ceil((H + spread) / tile_h), spread the widest of the segment's groups.
-long long fac_ctas(const mf_prf_table &tab, int64_t H, int64_t W, int seg);
+long long fac_ctas(const mf_prf_table &tab, int64_t H, int64_t W, int seg, int th);
+// Rows of a CTA's tile for this image: the plan's, or fewer when the image
+// would leave SMs without a CTA.
+int fac_tile_rows(const mf_prf_table &tab, int64_t H, int64_t W);
 struct FacBatchItem {
     FacParams p;
     long long cta_begin;  // first entry of this search in the batch's work list

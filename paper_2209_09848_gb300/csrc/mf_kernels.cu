@@ -64,20 +64,21 @@ __device__ __forceinline__ float to_f32<__half>(__half v) { return __half2float(
 __global__ void k_lambda(const float *__restrict__ sigma, const uint8_t *__restrict__ mask, int64_t H,
                          int64_t W, int64_t pad, int64_t lw, int64_t lh, float *__restrict__ lam,
                          unsigned int *lmax_bits) {
-    const int64_t n = lw * lh;
     float vmax = 0.f;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t yy = i / lw - pad, xx = i % lw - pad;
-        float v = 0.f;
-        if (yy >= 0 && yy < H && xx >= 0 && xx < W) {
-            const int64_t q = yy * W + xx;
-            const float s = sigma[q];
-            const bool m = mask ? (mask[q] != 0) : false;
-            if (!m && s > 0.f && isfinite(s)) v = (float)(1.0 / ((double)s * (double)s));
+    for (int64_t row = blockIdx.y; row < lh; row += gridDim.y)
+        for (int64_t col = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; col < lw;
+             col += (int64_t)gridDim.x * blockDim.x) {
+            const int64_t yy = row - pad, xx = col - pad;
+            float v = 0.f;
+            if (yy >= 0 && yy < H && xx >= 0 && xx < W) {
+                const int64_t q = yy * W + xx;
+                const float s = sigma[q];
+                const bool m = mask ? (mask[q] != 0) : false;
+                if (!m && s > 0.f && isfinite(s)) v = (float)(1.0 / ((double)s * (double)s));
+            }
+            lam[row * lw + col] = v;
+            vmax = fmaxf(vmax, v);
         }
-        lam[i] = v;
-        vmax = fmaxf(vmax, v);
-    }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) vmax = fmaxf(vmax, __shfl_xor_sync(0xffffffffu, vmax, o));
     if ((threadIdx.x & 31) == 0 && vmax > 0.f) atomicMax(lmax_bits, __float_as_uint(vmax));
@@ -259,37 +260,57 @@ __global__ void __launch_bounds__(256) k_denominator(const float *__restrict__ l
     }
 }
 
-// The same sums from a staged box.  A CTA owns `th` rows x kDenBoxCols start
-// pixels of one trajectory k: it copies the lambda box its start pixels
-// reach through G_k (rows dy0 .., columns x0 .. of the box, plus the tile),
-// G_k's weights and its runs into shared memory.  A thread then owns NO
-// consecutive start pixels of one tile row and slides an NO-wide register
-// window along each run, so that every 128-bit read of lambda feeds 4 NO
-// FMAs.  A warp covers 8 rows x 4 NO columns: the 8 threads of a quarter
-// warp hold the same columns of 8 consecutive rows, which an odd row pitch
-// (in 16-byte chunks) puts in 8 distinct bank groups, so the reads are
-// conflict-free at plain row-major addresses (base + chunk, no per-read
-// index arithmetic).  Same FP32 products, same FP64 accumulation as
-// k_denominator.
-template <int NO>
-__global__ void __launch_bounds__(32 * kDenBoxCols / NO) k_den_box(
+// One run of N chunks (4 taps each) for NO start pixels: every index is known
+// at compile time.
+template <int N, int NO>
+__device__ __forceinline__ void den_run(const float4 *row, const float4 *wp, float (&a)[NO]) {
+    float v[4 * (N + NO / 4)];
+#pragma unroll
+    for (int q = 0; q < N + NO / 4; q++) {
+        const float4 x = row[q];
+        v[4 * q] = x.x; v[4 * q + 1] = x.y; v[4 * q + 2] = x.z; v[4 * q + 3] = x.w;
+    }
+#pragma unroll
+    for (int ch = 0; ch < N; ch++) {
+        const float4 w4 = wp[ch];
+        const float w[4] = {w4.x, w4.y, w4.z, w4.w};
+#pragma unroll
+        for (int i = 0; i < 4; i++)
+#pragma unroll
+            for (int c = 0; c < NO; c++) a[c] = fmaf(w[i], v[4 * ch + i + c], a[c]);
+    }
+}
+
+// The same sums from a staged box.  A CTA owns `th` rows x C start pixels of
+// one trajectory k: it copies the lambda box its start pixels reach through G_k
+// (rows dy0 .., columns x0 .. of the box, plus the tile), G_k's weights and its
+// runs into shared memory.  A thread then owns NO consecutive start pixels of
+// one tile row and slides an NO-wide register window along each run, so that
+// every 128-bit read of lambda feeds 4 NO FMAs.  A warp covers 8 rows x 4 NO
+// columns: the 8 threads of a quarter warp hold the same columns of 8
+// consecutive rows, which an odd row pitch (in 16-byte chunks) puts in 8
+// distinct bank groups, so the reads are conflict-free at plain row-major
+// addresses (base + chunk, no per-read index arithmetic).  Same FP32 products,
+// same FP64 accumulation as k_denominator; the partials are widened by bits (a
+// conversion would cost a second FP64 operation each).
+template <int NO, int C>
+__global__ void __launch_bounds__(32 * C / NO, 256 / C) k_den_box(
     const float *__restrict__ lam, int64_t lw, int64_t lh, int64_t pad, const RunRec *__restrict__ runs,
     const int32_t *__restrict__ run_off, const float *__restrict__ wts, const DenBox *__restrict__ boxes, int K,
     int64_t H, int64_t W, int nbx, int th, float *__restrict__ isd) {
-    static_assert(NO % 4 == 0 && kDenBoxCols % (4 * NO) == 0, "whole chunks, whole warps per 8 rows");
-    constexpr int WR = kDenBoxCols / (4 * NO);  // warps per 8 tile rows
-    constexpr int S = NO / 4 + 1;                // window slots of 4 values
+    static_assert(NO % 4 == 0 && C % (4 * NO) == 0, "whole chunks, whole warps per 8 rows");
+    constexpr int WR = C / (4 * NO);  // warps per 8 tile rows
     extern __shared__ __align__(16) float4 dsm[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     // tile row y and first column xs of this thread's NO start pixels
     const int y = 8 * (warp / WR) + (lane & 7), xs = 4 * NO * (warp % WR) + NO * (lane >> 3);
     const int64_t py = (int64_t)(blockIdx.x / nbx) * th + y;
-    const int64_t px0 = (int64_t)(blockIdx.x % nbx) * kDenBoxCols;
+    const int64_t px0 = (int64_t)(blockIdx.x % nbx) * C;
     const int64_t P = H * W;
     const bool vec = (W & 3) == 0;  // rows (and planes) start on 16-byte boundaries
     for (int k = blockIdx.y; k < K; k += gridDim.y) {
         const DenBox bx = boxes[k];
-        const int R = th + bx.rows - 1, NC = (kDenBoxCols + bx.cols) / 4, PC = den_pitch(bx.cols);
+        const int R = th + bx.rows - 1, NC = (C + bx.cols) / 4, PC = den_pitch(bx.cols, C);
         const int r0 = run_off[k], nr = run_off[k + 1] - r0;
         float4 *wsm = dsm + (size_t)R * PC;                           // weights after the box
         RunRec *rsm = reinterpret_cast<RunRec *>(wsm + bx.nw / 4);    // then the runs
@@ -304,9 +325,15 @@ __global__ void __launch_bounds__(32 * kDenBoxCols / NO) k_den_box(
         }
         for (int i = threadIdx.x; i < bx.nw / 4; i += blockDim.x)
             wsm[i] = __ldg(reinterpret_cast<const float4 *>(wts + bx.w0) + i);
-        for (int i = threadIdx.x; i < nr; i += blockDim.x) rsm[i] = runs[r0 + i];
+        // a run's first chunk and weights relative to the box
+        for (int i = threadIdx.x; i < nr; i += blockDim.x) {
+            RunRec rr = runs[r0 + i];
+            rr.dy = (rr.dy - bx.dy0) * PC + (rr.x0 - bx.x0) / 4;
+            rr.woff = (rr.woff - bx.w0) / 4;
+            rsm[i] = rr;
+        }
         __syncthreads();
-        if (py >= H) continue;
+        if (py >= H || px0 + xs >= W) continue;
         double d[NO];
         float a[NO];
 #pragma unroll
@@ -314,43 +341,29 @@ __global__ void __launch_bounds__(32 * kDenBoxCols / NO) k_den_box(
             d[c] = 0.0;
             a[c] = 0.f;
         }
+        const float4 *mine = dsm + y * PC + xs / 4;
         int taps = 0;
         for (int r = 0; r < nr; r++) {
             const RunRec rr = rsm[r];
-            // the thread's first chunk of the run
-            const float4 *row = dsm + (size_t)(y + rr.dy - bx.dy0) * PC + (rr.x0 - bx.x0 + xs) / 4;
-            const float4 *wp = wsm + (rr.woff - bx.w0) / 4;
-            // window of NO + 4 lambda values in S float4 slots that rotate:
-            // chunk ch (4 taps) uses slot ch mod S onwards and, before its
-            // FMAs, loads the slot S - 1 ahead; unrolled by S so that every
-            // register index is static
-            float v[4 * S];
-#pragma unroll
-            for (int q = 0; q < S - 1; q++) {
-                const float4 pq = row[q];
-                v[4 * q] = pq.x; v[4 * q + 1] = pq.y; v[4 * q + 2] = pq.z; v[4 * q + 3] = pq.w;
-            }
-            for (int ch = 0; ch < rr.nch; ch += S) {
-#pragma unroll
-                for (int u = 0; u < S; u++) {
-                    if (ch + u < rr.nch) {
-                        const float4 pn = row[ch + u + S - 1];
-                        const int ns = ((u + S - 1) % S) * 4;  // slot receiving columns 4 (ch + u + S - 1) ..
-                        v[ns] = pn.x; v[ns + 1] = pn.y; v[ns + 2] = pn.z; v[ns + 3] = pn.w;
-                        const float4 w4 = wp[ch + u];
-                        const float w[4] = {w4.x, w4.y, w4.z, w4.w};
-#pragma unroll
-                        for (int i = 0; i < 4; i++)
-#pragma unroll
-                            for (int c = 0; c < NO; c++) a[c] = fmaf(w[i], v[(4 * u + i + c) % (4 * S)], a[c]);
-                    }
+            const float4 *row = mine + rr.dy, *wp = wsm + rr.woff;
+            // a slow mover's runs have two to four chunks
+            switch (rr.nch) {
+                case 1: den_run<1, NO>(row, wp, a); break;
+                case 2: den_run<2, NO>(row, wp, a); break;
+                case 3: den_run<3, NO>(row, wp, a); break;
+                case 4: den_run<4, NO>(row, wp, a); break;
+                case 5: den_run<5, NO>(row, wp, a); break;
+                default: {
+                    int ch = 0;
+                    for (; ch + 4 <= rr.nch; ch += 4) den_run<4, NO>(row + ch, wp + ch, a);
+                    for (; ch < rr.nch; ch++) den_run<1, NO>(row + ch, wp + ch, a);
                 }
             }
             taps += rr.nch * 4;
             if (taps >= kDenTaps) {
 #pragma unroll
                 for (int c = 0; c < NO; c++) {
-                    d[c] += (double)a[c];
+                    d[c] += widen(a[c]);
                     a[c] = 0.f;
                 }
                 taps = 0;
@@ -359,8 +372,9 @@ __global__ void __launch_bounds__(32 * kDenBoxCols / NO) k_den_box(
         float o[NO];
 #pragma unroll
         for (int c = 0; c < NO; c++) {
-            const double dd = d[c] + (double)a[c];
-            o[c] = dd > 0.0 ? rsqrtf((float)dd) : 0.f;
+            const double dd = d[c] + widen(a[c]);
+            const long long bits = __double_as_longlong(dd);  // dd > 0, by its bits (NaN is not)
+            o[c] = bits > 0 && bits <= 0x7FF0000000000000ll ? rsqrtf((float)dd) : 0.f;
         }
         const int64_t px = px0 + xs;
         float *dst = isd + (int64_t)k * P + py * W + px;
@@ -866,7 +880,31 @@ int profile_read(mf_profile *out, int reset) {
 
 namespace {
 
-// Inverse variance, weighted stack, denominator and a cleared key buffer.
+// Columns of a staged-denominator tile for images W wide: the widest of 256,
+// 128, 64, 32 unless a narrower one wastes less.  A tile's cost is its start
+// pixels (those past W too) times G_k's taps, plus the lambda values it stages
+// (about 6 FMAs' worth each); the narrower the tile, the more of these per
+// start pixel.  301 x 277, 54 trajectories, 231 taps each: 217 us with 256
+// columns (512 of them for 277), 99 with 32 (the loop by chunk counts and the
+// halved FP64 work included: 2048^2, 100 trajectories, 256 columns as before,
+// 17.2 -> 16.1 ms).
+int den_tile_cols(const mf_prf_table &tab, int64_t W) {
+    const double taps = (double)tab.g_nnz / tab.K;
+    int best = 256;
+    double least = 0.0;
+    for (int C = 256; C >= 32; C /= 2) {
+        const double stage = (1.0 + (double)tab.den_cols / C) * (1.0 + (double)tab.den_rows / tab.den_th);
+        const double cost = (double)((W + C - 1) / C * C) * (taps + 6.0 * stage);
+        if (C == 256 || cost < least) {
+            best = C;
+            least = cost;
+        }
+    }
+    return best;
+}
+
+// Inverse variance, weighted stack, denominator and (general numerator) a
+// cleared key buffer.
 int enqueue_pre(const SearchArgs &a, cudaStream_t stream, char *err, size_t errlen) {
     const mf_stack &st = *a.stack;
     const mf_prf_table &tab = *a.tab;
@@ -887,8 +925,11 @@ int enqueue_pre(const SearchArgs &a, cudaStream_t stream, char *err, size_t errl
     }
     {
         LaunchScope ls(kKLambda, stream);
-        k_lambda<<<grid_for(L.lam_w * L.lam_h, 256), 256, 0, stream>>>(a.sigma, a.mask, H, W, L.pad, L.lam_w,
-                                                                        L.lam_h, lam, lmax);
+        // rows and columns by grid dimension (no 64-bit division per pixel); a
+        // few blocks per SM, since every warp ends in an atomic maximum
+        const int64_t gx = (L.lam_w + 127) / 128, gy = std::max<int64_t>(1, std::min(L.lam_h, 152 * 16 / gx));
+        const dim3 grid((unsigned)std::min<int64_t>(gx, 65535), (unsigned)gy);
+        k_lambda<<<grid, 128, 0, stream>>>(a.sigma, a.mask, H, W, L.pad, L.lam_w, L.lam_h, lam, lmax);
     }
     MF_CHECK_LAUNCH("k_lambda");
 
@@ -919,21 +960,24 @@ int enqueue_pre(const SearchArgs &a, cudaStream_t stream, char *err, size_t errl
     }
     MF_CHECK_LAUNCH("k_weight");
     if (tab.den_th > 0) {
-        // staged: one CTA per (tile of den_th x 256 start pixels, trajectory)
-        const int th = tab.den_th;
-        const int nbx = (int)((W + kDenBoxCols - 1) / kDenBoxCols);
+        // staged: one CTA per (tile of den_th x C start pixels, trajectory)
+        const int th = tab.den_th, C = den_tile_cols(tab, W);
+        const size_t smem = den_box_smem(th, tab.den_rows, tab.den_cols, tab.den_nw, tab.den_nr, C);
+        const auto kern = C == 256   ? k_den_box<kDenOut, 256>
+                          : C == 128 ? k_den_box<kDenOut, 128>
+                          : C == 64  ? k_den_box<kDenOut, 64>
+                                     : k_den_box<kDenOut, 32>;
+        const int nbx = (int)((W + C - 1) / C);
         const int nby = (int)((H + th - 1) / th);
         dim3 grid((unsigned)(nbx * nby), (unsigned)std::min(tab.K, 65535));
-        cudaError_t ea = cudaFuncSetAttribute(k_den_box<kDenOut>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              (int)tab.den_smem);
+        cudaError_t ea = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemAllow);
         if (ea != cudaSuccess) {
             snprintf(err, errlen, "cudaFuncSetAttribute(k_den_box): %s", cudaGetErrorString(ea));
             return (int)ea;
         }
         LaunchScope ls(kKDenominator, stream);
-        k_den_box<kDenOut><<<grid, th * kDenBoxCols / kDenOut, tab.den_smem, stream>>>(
-            lam, L.lam_w, L.lam_h, L.pad, tab.d_runs, tab.d_run_off, tab.d_wts, tab.d_boxes, tab.K, H, W, nbx, th,
-            isd);
+        kern<<<grid, th * C / kDenOut, smem, stream>>>(lam, L.lam_w, L.lam_h, L.pad, tab.d_runs, tab.d_run_off,
+                                                       tab.d_wts, tab.d_boxes, tab.K, H, W, nbx, th, isd);
         MF_CHECK_LAUNCH("k_den_box");
     } else {
         const int nbx = (int)((W + kDenCols - 1) / kDenCols);
@@ -944,7 +988,11 @@ int enqueue_pre(const SearchArgs &a, cudaStream_t stream, char *err, size_t errl
                                                 W, nbx, isd);
         MF_CHECK_LAUNCH("k_denominator");
     }
-    cudaError_t e = cudaMemsetAsync(keys, 0, (size_t)P * sizeof(unsigned long long), stream);
+    // the general numerator merges its maxima into cleared keys; the factored
+    // one has none
+    const cudaError_t e = tab.plan.kernel == 2
+                              ? cudaSuccess
+                              : cudaMemsetAsync(keys, 0, (size_t)P * sizeof(unsigned long long), stream);
     if (e != cudaSuccess) {
         snprintf(err, errlen, "cudaMemsetAsync: %s", cudaGetErrorString(e));
         return (int)e;
@@ -992,9 +1040,9 @@ int numerator_params(const SearchArgs &a, CUtensorMap *map, NumParams *np, int *
     return 0;
 }
 
-// Tensor map and parameters of the factored numerator; *nblocks = CTAs.
-int fac_params(const SearchArgs &a, CUtensorMap *map, FacParams *fp, long long *nblocks, char *err,
-               size_t errlen) {
+// Tensor map and parameters of the factored numerator with tiles of `th` rows
+// (the plan's, or fewer).
+int fac_params(const SearchArgs &a, int th, CUtensorMap *map, FacParams *fp, char *err, size_t errlen) {
     const mf_stack &st = *a.stack;
     const mf_prf_table &tab = *a.tab;
     const Plan &pl = tab.plan;
@@ -1007,7 +1055,8 @@ int fac_params(const SearchArgs &a, CUtensorMap *map, FacParams *fp, long long *
     const bool y16 = L.ybytes == 2;
     cuuint64_t dims[3] = {(cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)T};
     cuuint64_t strides[2] = {(cuuint64_t)L.y_pitch * L.ybytes, (cuuint64_t)(H * L.y_pitch * L.ybytes)};
-    cuuint32_t box[3] = {(cuuint32_t)(y16 ? fac_rpitch16(pl.f_tw) : fac_rpitch(pl.f_tw)), (cuuint32_t)pl.f_bh, 1};
+    cuuint32_t box[3] = {(cuuint32_t)(y16 ? fac_rpitch16(pl.f_tw) : fac_rpitch(pl.f_tw)),
+                         (cuuint32_t)(pl.f_bh - (pl.f_th - th)), 1};
     cuuint32_t estr[3] = {1, 1, 1};
     const CUtensorMapDataType ty = !y16 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32
                                         : (st.dtype == MF_BF16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16
@@ -1032,17 +1081,17 @@ int fac_params(const SearchArgs &a, CUtensorMap *map, FacParams *fp, long long *
     fp->G = pl.G;
     fp->kt = pl.f_kt;
     fp->npl = pl.f_planes;
-    fp->th = pl.f_th;
-    fp->bh = pl.f_bh;
+    fp->th = th;
+    fp->dth = pl.f_th - th;
+    fp->bh = pl.f_bh - fp->dth;
     fp->ns = pl.f_ns;
     fp->S = pl.f_seg;
     fp->seg = 0;
     fp->K = tab.K;
-    fp->warps = pl.warps();
+    fp->warps = pl.warps_at(th);
     fp->H = H;
     fp->W = W;
     fp->tiles_x = (int)((W + pl.f_tw - 1) / pl.f_tw);
-    *nblocks = fac_ctas(tab, H, W, 0);
     return 0;
 }
 
@@ -1106,8 +1155,8 @@ int launch_search(const SearchArgs &a, char *err, size_t errlen) {
     CUtensorMap map;
     if (pl.kernel == 2) {
         FacParams fp;
-        long long nblocks = 0;
-        rc = fac_params(a, &map, &fp, &nblocks, err, errlen);
+        const int th = fac_tile_rows(*a.tab, a.stack->H, a.stack->W);
+        rc = fac_params(a, th, &map, &fp, err, errlen);
         if (rc) return rc;
         // one launch per time segment, in order: segment 0 stores the
         // numerator plane, the later ones add to it
@@ -1115,8 +1164,8 @@ int launch_search(const SearchArgs &a, char *err, size_t errlen) {
             fp.seg = j;
             LaunchScope ls(kKNumerator, stream);
             rc = fac_enqueue(&map, fp, pl.f_tw, pl.f_taps, a.L.ybytes == 2 ? a.stack->dtype : MF_F32,
-                             pl.launch_warps(), pl.smem(), fac_ctas(*a.tab, a.stack->H, a.stack->W, j), stream, err,
-                             errlen);
+                             (fp.warps + 3) / 4 * 4, pl.smem_at(th), fac_ctas(*a.tab, a.stack->H, a.stack->W, j, th),
+                             stream, err, errlen);
             if (rc) return rc;
         }
         return enqueue_finalize(a, stream, err, errlen);
@@ -1162,6 +1211,7 @@ struct BatchDevice {
     // width, with as many warps and as much shared memory as its largest
     // layout needs
     struct FacGroup {
+        int chain = 0;             // (tile width, element type): chains are independent of each other
         int tw = 32;
         int etype = MF_F32;        // element type of the weighted stacks
         int seg = 0;               // time segment (groups run in segment order)
@@ -1171,6 +1221,7 @@ struct BatchDevice {
         int warps = 0;
     };
     std::vector<FacGroup> fac;
+    std::vector<int> item_chain;  // the chain of each search, -1: general numerator
     CUtensorMap *d_fmaps = nullptr;
     FacBatchItem *d_fitems = nullptr;
     std::vector<FacBatchItem> h_fitems;  // the same, passed by value to each launch
@@ -1234,32 +1285,43 @@ int batch_build(const SearchArgs *items, int n, BatchDevice **out, char *err, si
     int max_seg = 0;
     for (int i = 0; i < n; i++)
         if (items[i].tab->plan.kernel == 2) max_seg = std::max(max_seg, items[i].tab->plan.f_seg);
+    // searches whose work entries take longest first, so that a launch ends on
+    // short ones (an entry's time goes with its frames and its warps' rows)
+    std::vector<int> by_time(n);
+    for (int i = 0; i < n; i++) by_time[i] = i;
+    auto entry = [&](int i) {
+        const Plan &pl = items[i].tab->plan;
+        return pl.kernel == 2 ? (double)items[i].stack->T / pl.f_seg * (pl.warps() + 8) : 0.0;
+    };
+    std::stable_sort(by_time.begin(), by_time.end(), [&](int x, int y) { return entry(x) > entry(y); });
+    b->item_chain.assign(n, -1);
     // one persistent launch per (segment, tile width, element type of the
     // weighted stack)
     for (int j = 0; j < max_seg; j++) {
         for (int tw : {32, 64})
         for (int et : {(int)MF_F32, (int)MF_BF16, (int)MF_F16}) {
             BatchDevice::FacGroup grp;
+            grp.chain = (tw == 64 ? 3 : 0) + et;
             grp.tw = tw;
             grp.etype = et;
             grp.seg = j;
             grp.first = (int)fitems.size();
-            for (int i = 0; i < n; i++) {
+            for (const int i : by_time) {
                 const Plan &pl = items[i].tab->plan;
                 const int item_et = items[i].L.ybytes == 2 ? items[i].stack->dtype : MF_F32;
                 if (pl.kernel != 2 || pl.f_tw != tw || item_et != et || j >= pl.f_seg) continue;
                 CUtensorMap m;
                 FacBatchItem fi;
                 std::memset(&fi, 0, sizeof fi);
-                long long nblocks = 0;
-                int rc = fac_params(items[i], &m, &fi.p, &nblocks, err, errlen);
+                int rc = fac_params(items[i], pl.f_th, &m, &fi.p, err, errlen);
                 if (rc) {
                     batch_free(b);
                     return rc;
                 }
+                b->item_chain[i] = grp.chain;
                 fi.p.seg = j;
                 fi.cta_begin = grp.total;
-                grp.total += fac_ctas(*items[i].tab, items[i].stack->H, items[i].stack->W, j);
+                grp.total += fac_ctas(*items[i].tab, items[i].stack->H, items[i].stack->W, j, pl.f_th);
                 grp.smem = std::max(grp.smem, pl.smem());
                 grp.warps = std::max(grp.warps, pl.launch_warps());
                 fmaps.push_back(m);
@@ -1351,13 +1413,6 @@ int batch_enqueue(BatchDevice *b, const SearchArgs *items, int n, void *stream_v
         snprintf(err, errlen, "batch join: %s", cudaGetErrorString(e));
         return (int)e;
     }
-    for (const auto &grp : b->groups) {
-        const int grid = (int)std::min<long long>(grp.total, (long long)b->sms);
-        LaunchScope ls(kKNumerator, stream);
-        pick_numerator_batch(grp.shape)<<<grid, kWarps * 32, grp.smem, stream>>>(
-            b->d_maps + grp.first, b->d_items + grp.first, grp.count, grp.total, b->d_counters + grp.shape);
-        MF_CHECK_LAUNCH("k_numerator_batch");
-    }
     if (!b->fac.empty()) {
         e = cudaMemsetAsync(b->d_fcounters, 0, b->fac.size() * sizeof(unsigned long long), stream);
         if (e != cudaSuccess) {
@@ -1365,18 +1420,44 @@ int batch_enqueue(BatchDevice *b, const SearchArgs *items, int n, void *stream_v
             return (int)e;
         }
     }
+    // Factored searches: the launches of one tile width and element type follow
+    // each other (segments in order, then the finalisation), those of different
+    // ones run side by side, so that one chain's next CTAs take the SMs that the
+    // last work entries of another leave.  General ones stay on `stream`.
+    e = cudaEventRecord(b->fork, stream);
+    for (int s = 0; s < BatchDevice::kSide && e == cudaSuccess; s++) e = cudaStreamWaitEvent(b->side[s], b->fork, 0);
+    if (e != cudaSuccess) {
+        snprintf(err, errlen, "batch fork: %s", cudaGetErrorString(e));
+        return (int)e;
+    }
+    auto lane = [&](int chain) { return chain < 0 ? stream : b->side[chain % BatchDevice::kSide]; };
+    for (const auto &grp : b->groups) {
+        const int grid = (int)std::min<long long>(grp.total, (long long)b->sms);
+        LaunchScope ls(kKNumerator, stream);
+        pick_numerator_batch(grp.shape)<<<grid, kWarps * 32, grp.smem, stream>>>(
+            b->d_maps + grp.first, b->d_items + grp.first, grp.count, grp.total, b->d_counters + grp.shape);
+        MF_CHECK_LAUNCH("k_numerator_batch");
+    }
     for (size_t gi = 0; gi < b->fac.size(); gi++) {
         const auto &grp = b->fac[gi];
         const int grid = (int)std::min<long long>(grp.total, (long long)b->sms);
-        LaunchScope ls(kKNumerator, stream);
+        LaunchScope ls(kKNumerator, lane(grp.chain));
         int rc = fac_batch_enqueue(b->d_fmaps + grp.first, b->h_fitems.data() + grp.first, grp.count, grp.total,
-                                   b->d_fcounters + gi, grp.tw, grp.etype, grp.warps, grp.smem, grid, stream, err,
-                                   errlen);
+                                   b->d_fcounters + gi, grp.tw, grp.etype, grp.warps, grp.smem, grid,
+                                   lane(grp.chain), err, errlen);
         if (rc) return rc;
     }
     for (int i = 0; i < n; i++) {
-        int rc = enqueue_finalize(items[i], stream, err, errlen);
+        int rc = enqueue_finalize(items[i], lane(b->item_chain[i]), err, errlen);
         if (rc) return rc;
+    }
+    for (int s = 0; s < BatchDevice::kSide && e == cudaSuccess; s++) {
+        e = cudaEventRecord(b->join[s], b->side[s]);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(stream, b->join[s], 0);
+    }
+    if (e != cudaSuccess) {
+        snprintf(err, errlen, "batch join: %s", cudaGetErrorString(e));
+        return (int)e;
     }
     return 0;
 }

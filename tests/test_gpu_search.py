@@ -428,3 +428,47 @@ def test_shift_stack_single_tap_equals_batch(mf):
     assert torch.equal(smax, bmax) and torch.equal(amax, bamax)
     assert mf.prf_table_create(vx, vy, T).info()["taps"] == 5
 
+
+
+@pytest.mark.parametrize("W", [31, 32, 33, 65, 96, 129, 200, 257])
+def test_denominator_tile_widths(mf, oracle, W):
+    # the staged denominator's tile columns follow the image's width (32 to
+    # 256); runs of one to many chunks, from slow and fast movers
+    from paper_2209_09848_gb300 import synth
+    T, H = 21, 43
+    c = synth.small_case(T, H, W, 300 + W, mask_frac=0.02, movers=1)
+    vx = np.array([0.0, 0.0, 0.3, -0.3, 1.7])
+    vy = np.array([0.0, 0.6, 0.1, -0.4, 0.2])
+    table = mf.prf_table_create(vx, vy, T)
+    assert table.info()["den_tile_h"] > 0
+    sh, tp = oracle.trajectory_table(vx, vy, T)
+    lam = oracle.inverse_variance(c["sigma"], c["mask"])
+    N, D = oracle.search_full(c["res"], lam, sh, tp)
+    smax, amax, sall = _run(mf, c["res"], c["sigma"], c["mask"], table)
+    check_search(smax, amax, sall, N, D, oracle, label="W %d" % W)
+
+
+@pytest.mark.parametrize("H,W,layout", [
+    (40, 70, dict(group=5, tile_h=128)), (33, 32, dict(group=4, tile_h=160)), (130, 64, dict(group=2, tile_h=224)),
+    (100, 130, dict(group=3, tile_h=96, tile_w=64)), (97, 31, dict(group=1, tile_h=224, segments=2)),
+])
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_small_images_take_shorter_tiles(mf, oracle, H, W, layout, dtype):
+    # tiles shorter than the plan's on images with few of them: windows and row
+    # passes shrink alike; several record chunks and frame blocks
+    from paper_2209_09848_gb300 import synth
+    T = 37
+    c = synth.small_case(T, H, W, H + W, mask_frac=0.01, movers=2)
+    vx, vy = synth.velocity_grid(2, 5, -0.4, 0.4)
+    table = mf.prf_table_create(vx, vy, T, kernel=2, **layout)
+    sh, tp = oracle.trajectory_table(vx, vy, T)
+    lam = oracle.inverse_variance(c["sigma"], c["mask"])
+    if dtype == "f32":
+        N, D = oracle.search_full(c["res"], lam, sh, tp)
+        smax, amax, sall = _run(mf, c["res"], c["sigma"], c["mask"], table)
+    else:
+        deq = torch.from_numpy(c["res"]).to(torch.bfloat16).float().numpy()
+        y16, beta = oracle.weighted_stack16(deq, c["sigma"], c["mask"], None, "bf16")
+        N, D = oracle.search_weighted(y16, beta, lam, sh, tp)
+        smax, amax, sall = _run(mf, deq, c["sigma"], c["mask"], table, dtype=torch.bfloat16)
+    check_search(smax, amax, sall, N, D, oracle, label="%s %s" % ((H, W), layout))
