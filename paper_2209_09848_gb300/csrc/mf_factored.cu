@@ -51,6 +51,31 @@ using namespace dev;
 // why).  The CTA may have more warps than the search's layout uses (batched
 // searches share one launch): the extra warps take part in the row pass and
 // the barriers only.  `smem` is the CTA's 1024-aligned dynamic shared memory.
+// Shared memory by 32-bit address: the frame loop keeps its addresses in
+// registers, where C++ pointers into the dynamic array are formed again at every
+// access (with the row pass's fixed units below, 2.54e9 -> 2.35e9 instructions
+// on 1000 x 512^2 x 100 and 9.85 -> 9.42 ms; of a column pass by itself, 160
+// FMAs and 20 reads, the FP32 pipe reaches 70 % of its peak).  Volatile: they
+// stay on their side of the barriers.
+__device__ __forceinline__ float2 lds2(uint32_t a) {
+    float2 v;
+    asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(a));
+    return v;
+}
+__device__ __forceinline__ float4 lds4(uint32_t a) {
+    float4 v;
+    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(a));
+    return v;
+}
+__device__ __forceinline__ uint4 lds4u(uint32_t a) {
+    uint4 v;
+    asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a));
+    return v;
+}
+__device__ __forceinline__ void sts4(uint32_t a, float x, float y, float z, float w) {
+    asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(a), "f"(x), "f"(y), "f"(z), "f"(w));
+}
+
 // Values of a staged window: FP32, or the 16-bit types of a bf16 / fp16
 // weighted stack, converted exactly to FP32 as they are read.
 template <typename E>
@@ -58,8 +83,8 @@ struct Win;
 template <>
 struct Win<float> {
     static constexpr int kPer = 4;  // values per 128-bit load
-    static __device__ __forceinline__ void load(const void *p, float *v) {
-        const float4 x = *reinterpret_cast<const float4 *>(p);
+    static __device__ __forceinline__ void load(uint32_t p, float *v) {
+        const float4 x = lds4(p);
         v[0] = x.x;
         v[1] = x.y;
         v[2] = x.z;
@@ -70,8 +95,8 @@ struct Win<float> {
 template <>
 struct Win<__nv_bfloat16> {
     static constexpr int kPer = 8;
-    static __device__ __forceinline__ void load(const void *p, float *v) {
-        const uint4 x = *reinterpret_cast<const uint4 *>(p);
+    static __device__ __forceinline__ void load(uint32_t p, float *v) {
+        const uint4 x = lds4u(p);
         const uint32_t w[4] = {x.x, x.y, x.z, x.w};
 #pragma unroll
         for (int i = 0; i < 4; i++) {  // a bf16 is the high half of the FP32 with the same value
@@ -84,8 +109,8 @@ struct Win<__nv_bfloat16> {
 template <>
 struct Win<__half> {
     static constexpr int kPer = 8;
-    static __device__ __forceinline__ void load(const void *p, float *v) {
-        const uint4 x = *reinterpret_cast<const uint4 *>(p);
+    static __device__ __forceinline__ void load(uint32_t p, float *v) {
+        const uint4 x = lds4u(p);
         const uint32_t w[4] = {x.x, x.y, x.z, x.w};
 #pragma unroll
         for (int i = 0; i < 4; i++) {
@@ -102,13 +127,13 @@ struct Win<__half> {
 // aligned, dst = H(row, c0).  TAPS = 1 (single-tap footprints: the
 // shift-stack filter) keeps the centre tap only.
 template <int M, int TAPS, typename E>
-__device__ __forceinline__ void row_item(const E *__restrict__ src, float *__restrict__ dst, float ux0,
-                                         float ux1, float ux2, float ux3, float ux4) {
+__device__ __forceinline__ void row_item(uint32_t src, uint32_t dst, float ux0, float ux1, float ux2, float ux3,
+                                         float ux4) {
     constexpr int PER = Win<E>::kPer;
     constexpr int NL = (kFacItem + (TAPS == 1 ? 3 : 4) + M + PER - 1) / PER;  // 128-bit loads covering the inputs
     float v[PER * NL];
 #pragma unroll
-    for (int q = 0; q < NL; q++) Win<E>::load(src + PER * q, v + PER * q);
+    for (int q = 0; q < NL; q++) Win<E>::load(src + 16 * q, v + PER * q);
     float o[kFacItem];
 #pragma unroll
     for (int c = 0; c < kFacItem; c++) {
@@ -124,7 +149,7 @@ __device__ __forceinline__ void row_item(const E *__restrict__ src, float *__res
     }
 #pragma unroll
     for (int q = 0; q < kFacItem / 4; q++)
-        reinterpret_cast<float4 *>(dst)[q] = make_float4(o[4 * q], o[4 * q + 1], o[4 * q + 2], o[4 * q + 3]);
+        sts4(dst + 16 * q, o[4 * q], o[4 * q + 1], o[4 * q + 2], o[4 * q + 3]);
 }
 
 // The (group, tile) of CTA `cta` of the launch that computes segment p.seg,
@@ -255,17 +280,17 @@ __device__ __forceinline__ bool fac_tile(const CUtensorMap &ymap, const FacParam
     auto record = [&](int f) { return fb + (f & 15) * kBB; };
     // the column pass of one frame: its records at rec, its row-pass buffer at h
     const int lane_off = (32 * sub_y + 16 * rh) * HP + 32 * sub_x + 2 * cp;
-    auto column = [&](const unsigned char *rec, const float *h) {
-        const FacSlot *fs = reinterpret_cast<const FacSlot *>(rec + sizeof(FacHdr)) + slot;
-        const float4 u4 = *reinterpret_cast<const float4 *>(fs->uy);
-        const float2 u5 = *reinterpret_cast<const float2 *>(fs->uy + 4);  // u_y(2) and the row offset
+    const uint32_t slot_off = (uint32_t)(sizeof(FacHdr) + slot * sizeof(FacSlot));
+    auto column = [&](uint32_t rec, uint32_t h) {  // h: the lane's place in row 0 of the buffer
+        const float4 u4 = lds4(rec + slot_off);
+        const float2 u5 = lds2(rec + slot_off + 16);  // u_y(2) and the row offset
         const float u[5] = {u4.x, u4.y, u4.z, u4.w, u5.x};
-        const float *col = h + lane_off + __float_as_int(u5.y) * HP;
+        const uint32_t col = h + (uint32_t)(__float_as_int(u5.y) * (HP * 4));
         // taps b = B0 .. B1 of the footprint (all five, or the centre one)
         constexpr int B0 = 2 - TAPS / 2, B1 = 2 + TAPS / 2;
 #pragma unroll
         for (int i = B0; i < 16 + B1; i++) {
-            const float2 hv = *reinterpret_cast<const float2 *>(col + i * HP);
+            const float2 hv = lds2(col + i * (HP * 4));
 #pragma unroll
             for (int b = B0; b <= B1; b++) {
                 const int r = i - b;
@@ -297,44 +322,46 @@ __device__ __forceinline__ bool fac_tile(const CUtensorMap &ymap, const FacParam
             for (int r = 0; r < 32; r++) blk[r] += Win<E>::one(col + r * RP);
         }
     };
-    // the row passes of frames f0 (records rec0, window w0, buffer h0) and f0 +
-    // 1 (if `two`; records, window w1, buffer h1 likewise), in units of 32 rows
-    // x 16 columns, an item per lane: a unit has one frame, one column phase
-    // and one address stride, so its set-up is uniform over the warp
-    auto row_pair = [&](int f0, const unsigned char *rec0, const E *w0, const E *w1, float *h0, float *h1, bool two) {
-        const unsigned char *rec1 = rec0 + (two ? kBB : 0u);
-        const int rows0 = reinterpret_cast<const FacHdr *>(rec0)->nrows - p.dth;
-        const int rows1 = two ? reinterpret_cast<const FacHdr *>(rec1)->nrows - p.dth : 0;
-        const int n0 = ((rows0 + 31) >> 5) * NI, n1 = ((rows1 + 31) >> 5) * NI;
-        for (int it = nwarps - 1 - warp; it < n0 + n1; it += nwarps) {
-            const bool second = it >= n0;
-            const int j = second ? it - n0 : it, m = j % NI, row = (j / NI) * 32 + lane;
-            const float4 *hd = reinterpret_cast<const float4 *>(second ? rec1 : rec0);
-            const float4 ua = hd[1], ub = hd[2];  // u_x(-2 .. 1); u_x(2), 1 / nrows, column phase of 16-bit windows
-            if (row >= (second ? rows1 : rows0)) continue;
-            const E *src = (second ? w1 : w0) + row * RP + kFacItem * m;
-            float *dst = (second ? h1 : h0) + row * HP + kFacItem * m;
+    // The row passes of frames f0 (records rec0, window w0) and f0 + 1 (if `two`;
+    // the next records, window w1) into the buffers at h0 and the next one, in
+    // units of 32 rows x 16 columns, an item per lane.  Warps take the two
+    // frames alternately, the last warps first (those past the column passes'
+    // have no other work): a warp's frame, rows and columns are the same in
+    // every pair but for windows of more units than half the warps.
+    const int row_e = (nwarps - 1 - warp) & 1, row_u = (nwarps - 1 - warp) >> 1, row_n = nwarps >> 1;
+    auto row_pair = [&](int f0, uint32_t rec0, uint32_t w0, uint32_t w1, uint32_t h0, bool two) {
+        if (row_e && !two) return;
+        const uint32_t hd = rec0 + (row_e ? kBB : 0u), win = row_e ? w1 : w0;
+        const uint32_t hb = h0 + (row_e ? (uint32_t)(BH * HP * 4) : 0u);
+        const float2 ph = lds2(hd + 8);  // FacHdr.cofs, nrows
+        const int rows = __float_as_int(ph.y) - p.dth, cofs = __float_as_int(ph.x);
+        for (int u = row_u; 32 * (u / NI) < rows; u += row_n) {
+            const int m = u % NI, row = (u / NI) * 32 + lane;
+            const float4 ua = lds4(hd + 16), ub = lds4(hd + 32);  // u_x; u_x(2), 1 / nrows, phase of 16-bit windows
+            if (row >= rows) break;  // the last rows: no later unit has more of this lane's
+            const uint32_t src = win + (uint32_t)(row * RP + kFacItem * m) * (uint32_t)sizeof(E);
+            const uint32_t dst = hb + (uint32_t)(row * HP + kFacItem * m) * 4u;
             if constexpr (k16) {
                 // the taps carry the frame's scale of a 16-bit weighted stack
                 // (a power of two: u_x * beta is exact)
-                const float bt = p.beta ? p.beta[second ? f0 + 1 : f0] : 1.f;
+                const float bt = p.beta ? p.beta[f0 + row_e] : 1.f;
                 const float ux0 = ua.x * bt, ux1 = ua.y * bt, ux2 = ua.z * bt, ux3 = ua.w * bt, ux4 = ub.x * bt;
                 switch (__float_as_int(ub.z)) {
-                    case 0: row_item<0, TAPS>(src, dst, ux0, ux1, ux2, ux3, ux4); break;
-                    case 1: row_item<1, TAPS>(src, dst, ux0, ux1, ux2, ux3, ux4); break;
-                    case 2: row_item<2, TAPS>(src, dst, ux0, ux1, ux2, ux3, ux4); break;
-                    case 3: row_item<3, TAPS>(src, dst, ux0, ux1, ux2, ux3, ux4); break;
-                    case 4: row_item<4, TAPS>(src, dst, ux0, ux1, ux2, ux3, ux4); break;
-                    case 5: row_item<5, TAPS>(src, dst, ux0, ux1, ux2, ux3, ux4); break;
-                    case 6: row_item<6, TAPS>(src, dst, ux0, ux1, ux2, ux3, ux4); break;
-                    default: row_item<7, TAPS>(src, dst, ux0, ux1, ux2, ux3, ux4); break;
+                    case 0: row_item<0, TAPS, E>(src, dst, ux0, ux1, ux2, ux3, ux4); break;
+                    case 1: row_item<1, TAPS, E>(src, dst, ux0, ux1, ux2, ux3, ux4); break;
+                    case 2: row_item<2, TAPS, E>(src, dst, ux0, ux1, ux2, ux3, ux4); break;
+                    case 3: row_item<3, TAPS, E>(src, dst, ux0, ux1, ux2, ux3, ux4); break;
+                    case 4: row_item<4, TAPS, E>(src, dst, ux0, ux1, ux2, ux3, ux4); break;
+                    case 5: row_item<5, TAPS, E>(src, dst, ux0, ux1, ux2, ux3, ux4); break;
+                    case 6: row_item<6, TAPS, E>(src, dst, ux0, ux1, ux2, ux3, ux4); break;
+                    default: row_item<7, TAPS, E>(src, dst, ux0, ux1, ux2, ux3, ux4); break;
                 }
             } else {
-                switch (reinterpret_cast<const FacHdr *>(hd)->cofs) {
-                    case 0: row_item<0, TAPS>(src, dst, ua.x, ua.y, ua.z, ua.w, ub.x); break;
-                    case 1: row_item<1, TAPS>(src, dst, ua.x, ua.y, ua.z, ua.w, ub.x); break;
-                    case 2: row_item<2, TAPS>(src, dst, ua.x, ua.y, ua.z, ua.w, ub.x); break;
-                    default: row_item<3, TAPS>(src, dst, ua.x, ua.y, ua.z, ua.w, ub.x); break;
+                switch (cofs) {
+                    case 0: row_item<0, TAPS, E>(src, dst, ua.x, ua.y, ua.z, ua.w, ub.x); break;
+                    case 1: row_item<1, TAPS, E>(src, dst, ua.x, ua.y, ua.z, ua.w, ub.x); break;
+                    case 2: row_item<2, TAPS, E>(src, dst, ua.x, ua.y, ua.z, ua.w, ub.x); break;
+                    default: row_item<3, TAPS, E>(src, dst, ua.x, ua.y, ua.z, ua.w, ub.x); break;
                 }
             }
         }
@@ -420,8 +447,8 @@ __device__ __forceinline__ bool fac_tile(const CUtensorMap &ymap, const FacParam
             bool ready = mbar_wait(smem_u32(&bars[s]), par, 1, p.status);
             if (ready && two) ready = mbar_wait(smem_u32(&bars[s1]), par1, 1, p.status);
             if (ready)
-                row_pair(t, record(t), rwin + (size_t)s * SF * EPF, rwin + (size_t)s1 * SF * EPF, hbuf,
-                         hbuf + (size_t)BH * HP, two);
+                row_pair(t, smem_u32(record(t)), smem_u32(rwin + (size_t)s * SF * EPF),
+                         smem_u32(rwin + (size_t)s1 * SF * EPF), smem_u32(hbuf), two);
             if (__syncthreads_or(!ready)) {
                 bad = true;
                 break;
@@ -453,15 +480,19 @@ __device__ __forceinline__ bool fac_tile(const CUtensorMap &ymap, const FacParam
         }
     }
     int in_block = 0;  // frames in the current partial sums
+    // 32-bit addresses of the loop, formed once (volatile: not formed again)
+    uint32_t a_win = smem_u32(smem), a_h = smem_u32(hbuf), a_rec0 = smem_u32(fb), a_bar0 = smem_u32(bars);
+    asm volatile("" : "+r"(a_win), "+r"(a_h), "+r"(a_rec0), "+r"(a_bar0));
+    const uint32_t a_lane = (uint32_t)lane_off * 4u, st_b = (uint32_t)SF * 4u;
+    uint32_t rec = a_rec0 + (uint32_t)(t0 & 15) * kBB, h = a_h;
+    const uint32_t rec_end = a_rec0 + 16 * kBB, h_sum = 2 * a_h + 2u * (uint32_t)(BH * HP * 4);
     for (int t = t0; t < t1 && !QG; t += 2) {  // column passes (the loop is empty for QG); t is even
         const bool two = t + 1 < t1;
-        const int s1 = (s + 1 == NS) ? 0 : s + 1;
-        const uint32_t par1 = (s + 1 == NS) ? (par ^ 1u) : par;
-        bool ready = mbar_wait(smem_u32(&bars[s]), par, 1, p.status);
-        if (ready && two) ready = mbar_wait(smem_u32(&bars[s1]), par1, 1, p.status);
-        const unsigned char *rec = record(t);
-        // row-pass buffers 0, 1 and 2, 3 in turn
-        float *h0 = hbuf + (t & 2) * (BH * HP), *h1 = h0 + BH * HP;
+        const bool wrap = s + 1 == NS;
+        const int s1 = wrap ? 0 : s + 1;
+        const uint32_t par1 = wrap ? (par ^ 1u) : par;
+        bool ready = mbar_wait(a_bar0 + 8 * s, par, 1, p.status);
+        if (ready && two) ready = mbar_wait(a_bar0 + 8 * s1, par1, 1, p.status);
         if (TAPS == 1) {
             // the column passes read the stages themselves: they run before
             // the barrier that frees the stages for refilling
@@ -470,7 +501,7 @@ __device__ __forceinline__ bool fac_tile(const CUtensorMap &ymap, const FacParam
                 if (two) column_direct(t + 1, s1);
             }
         } else if (ready) {
-            row_pair(t, rec, rwin + s * (SF * EPF), rwin + s1 * (SF * EPF), h0, h1, two);
+            row_pair(t, rec, a_win + s * st_b, a_win + s1 * st_b, h, two);
         }
         if (__syncthreads_or(!ready)) {
             bad = true;
@@ -480,17 +511,17 @@ __device__ __forceinline__ bool fac_tile(const CUtensorMap &ymap, const FacParam
         if (threadIdx.x == 0) {
             fence_proxy_async();
             if (t + NS < t1) {
-                const FacHdr *fh = reinterpret_cast<const FacHdr *>(rec);
-                issue(t + NS, s, fh->next_roy, fh->next_rox);
+                const float2 nx = lds2(rec);  // next_roy, next_rox
+                issue(t + NS, s, __float_as_int(nx.x), __float_as_int(nx.y));
             }
             if (two && t + 1 + NS < t1) {
-                const FacHdr *fh = reinterpret_cast<const FacHdr *>(rec + kBB);
-                issue(t + 1 + NS, s1, fh->next_roy, fh->next_rox);
+                const float2 nx = lds2(rec + kBB);
+                issue(t + 1 + NS, s1, __float_as_int(nx.x), __float_as_int(nx.y));
             }
         }
         if (TAPS != 1 && active) {
-            column(rec, h0);
-            if (two) column(rec + kBB, h1);
+            column(rec, h + a_lane);
+            if (two) column(rec + kBB, h + a_lane + (uint32_t)(BH * HP * 4));
         }
         in_block += 2;
         if (in_block == kFrameBlock) {
@@ -504,6 +535,9 @@ __device__ __forceinline__ bool fac_tile(const CUtensorMap &ymap, const FacParam
         // advance two stages
         s = (s1 + 1 == NS) ? 0 : s1 + 1;
         par = (s1 + 1 == NS) ? (par1 ^ 1u) : par1;
+        h = h_sum - h;  // row-pass buffers 0, 1 and 2, 3 in turn
+        rec += 2 * kBB;
+        if (rec == rec_end) rec = a_rec0;
     }
     if (bad) {
         // let any copy still in flight land before the CTA's shared memory goes away
