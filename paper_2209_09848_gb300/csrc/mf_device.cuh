@@ -95,6 +95,25 @@ __device__ __forceinline__ void bulk_load(uint32_t dst, const void *src, uint32_
         : "memory");
 }
 
+// Programmatic dependent launches: a kernel lets the next one in its stream
+// start once all its CTAs have (or have ended), and a kernel waits for the one
+// before it to have completed, with everything it wrote.  Without that launch
+// attribute both do nothing.
+__device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// Loads of what the awaited kernel wrote: from L2 (a line that an earlier CTA
+// of this SM cached may be older), and in program order with the wait, which
+// loads through const __restrict__ pointers need not be.
+__device__ __forceinline__ void load_awaited(float &v, const float *p) {
+    asm volatile("ld.global.cg.f32 %0, [%1];" : "=f"(v) : "l"(p));
+}
+__device__ __forceinline__ void load_awaited(float4 &v, const float4 *p) {
+    asm volatile("ld.global.cg.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+                 : "l"(p));
+}
+
 // Order-preserving 64-bit key: larger SNR first, then smaller k.  Any valid
 // key is nonzero, so 0 means "no filter with D > 0".
 __device__ __forceinline__ unsigned long long pack_key(float snr, int k) {

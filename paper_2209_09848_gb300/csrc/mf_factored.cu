@@ -181,7 +181,7 @@ __device__ __forceinline__ bool fac_locate(const FacParams &p, int tw, long long
 // per frame the row pass, then one column pass per rounded y-phase present
 // (a plane over the whole window), then one add per (trajectory, pixel)
 // gathered from its phase's plane.
-template <int TW, int TAPS, typename E, bool QG = false>
+template <int TW, int TAPS, typename E, bool EARLY, bool QG = false>
 __device__ __forceinline__ bool fac_tile(const CUtensorMap &ymap, const FacParams &p, long long cta,
                                          unsigned char *smem) {
     static_assert(!QG || (TAPS == 5 && sizeof(E) == 4), "phase planes: five taps, FP32 stacks");
@@ -556,17 +556,35 @@ __device__ __forceinline__ bool fac_tile(const CUtensorMap &ymap, const FacParam
     // pixel is the tile pixel minus the trajectory's s_y at the segment's
     // first frame, and each is reached by one CTA of the launch
     const int64_t P = p.H * p.W;
+    if (EARLY && seg != 0) wait_previous();
     if (kk >= 0) {
         float *plane = p.plane + (size_t)kk * P;
-#pragma unroll
-        for (int r = 0; r < 32; r++) {
+        auto at = [&](int r) {
             const int64_t px = tile_x0 + 32 * sub_x + (TAPS == 1 ? lane : 2 * cp + (r & 1));
             const int64_t py = (int64_t)tile_y0 + 32 * sub_y + (TAPS == 1 ? r : 16 * rh + (r >> 1)) - ref;
-            if (py >= 0 && py < p.H && px < p.W) {
-                const int64_t q = py * p.W + px;
-                plane[q] = seg == 0 ? acc[r] + blk[r] : plane[q] + (acc[r] + blk[r]);
+            return py >= 0 && py < p.H && px < p.W ? py * p.W + px : (int64_t)-1;
+        };
+#pragma unroll
+        for (int r = 0; r < 32; r++) acc[r] += blk[r];
+        if (seg != 0) {
+            // the loads of 16 pixels before the first sum: one latency, not 16
+            // (three segments of 1000 x 2048^2 frames x 100 trajectories: 130.2
+            // ms of numerator, with a load before each sum 132.1)
+#pragma unroll
+            for (int h = 0; h < 32; h += 16) {
+                float before[16];
+#pragma unroll
+                for (int r = 0; r < 16; r++) {
+                    before[r] = 0.f;
+                    if (at(h + r) >= 0) load_awaited(before[r], plane + at(h + r));
+                }
+#pragma unroll
+                for (int r = 0; r < 16; r++) acc[h + r] = before[r] + acc[h + r];
             }
         }
+#pragma unroll
+        for (int r = 0; r < 32; r++)
+            if (at(r) >= 0) plane[at(r)] = acc[r];
     }
     // the barriers may be initialised again for this CTA's next tile
     if (threadIdx.x == 0)
@@ -574,12 +592,24 @@ __device__ __forceinline__ bool fac_tile(const CUtensorMap &ymap, const FacParam
     return true;
 }
 
+// A CTA that started early (see launch_after): segment 0 reads the weighted
+// stack, so the kernel before must have completed; a later segment follows
+// segment 0, which waited for it, and needs its predecessor only for the
+// numerator plane, in the epilogue.  What follows may start when every CTA is
+// here.
+__device__ __forceinline__ void start_early(const FacParams &p) {
+    if (p.seg == 0) wait_previous();
+    launch_dependents();
+}
+
 template <int TW, int TAPS, typename E>
 __global__ void __launch_bounds__(32 * kFacMaxWarps, 1)
     k_numerator_fac(const __grid_constant__ CUtensorMap ymap, const FacParams p) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char *smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
-    fac_tile<TW, TAPS, E>(ymap, p, (long long)blockIdx.x, smem);
+    start_early(p);
+    // ends after the segment before it in any case
+    if (!fac_tile<TW, TAPS, E, true>(ymap, p, (long long)blockIdx.x, smem)) wait_previous();
 }
 
 // The factored numerator with phase planes (phase-quantised banks).
@@ -588,7 +618,9 @@ __global__ void __launch_bounds__(32 * kFacMaxWarps, 1)
     k_numerator_fac_planes(const __grid_constant__ CUtensorMap ymap, const FacParams p) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char *smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
-    fac_tile<TW, 5, float, true>(ymap, p, (long long)blockIdx.x, smem);
+    start_early(p);
+    // ends after the segment before it in any case
+    if (!fac_tile<TW, 5, float, true, true>(ymap, p, (long long)blockIdx.x, smem)) wait_previous();
 }
 
 // Persistent factored numerator over a batch of searches: one CTA per SM
@@ -622,7 +654,7 @@ __global__ void __launch_bounds__(32 * kFacMaxWarps, 1)
         const FacParams &p = a.items[i].p;
         // the five-tap code: single-tap footprints give the same sums (zero
         // taps add exact zeros), so a batch of mixed tables needs one kernel
-        if (!fac_tile<TW, 5, E>(maps[i], p, w - a.items[i].cta_begin, smem)) break;
+        if (!fac_tile<TW, 5, E, false>(maps[i], p, w - a.items[i].cta_begin, smem)) break;
         __syncthreads();
     }
 }
@@ -636,6 +668,7 @@ __global__ void k_finalize_planes(const float *__restrict__ plane, const float *
                                   float *__restrict__ snr_max, int32_t *__restrict__ argmax,
                                   float *__restrict__ snr_all, const int *slot, int *global_status) {
     using VecT = typename std::conditional<V == 4, float4, float>::type;
+    wait_previous();
     // a failure of this search also goes into the device-wide word
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         const int s = *(const volatile int *)slot;
@@ -650,23 +683,36 @@ __global__ void k_finalize_planes(const float *__restrict__ plane, const float *
             best[v] = 0.f;
             arg[v] = -1;
         }
-#pragma unroll 4
-        for (int k = 0; k < K; k++) {
-            const VecT xv = reinterpret_cast<const VecT *>(plane + (int64_t)k * P)[i];
-            const VecT dv = reinterpret_cast<const VecT *>(isd + (int64_t)k * P)[i];
-            const float *x = reinterpret_cast<const float *>(&xv);
-            const float *d = reinterpret_cast<const float *>(&dv);
-            float snr[V];
+        // the loads of four filters before the first is used (the SNR cube's
+        // stores would hold them back otherwise)
+        constexpr int KB = 4;
+        for (int k0 = 0; k0 < K; k0 += KB) {
+            VecT xv[KB] = {}, dv[KB] = {};
 #pragma unroll
-            for (int v = 0; v < V; v++) {
-                snr[v] = x[v] * d[v];
-                if (d[v] > 0.f && (arg[v] < 0 || snr[v] > best[v])) {
-                    best[v] = snr[v];
-                    arg[v] = k;
+            for (int j = 0; j < KB; j++)
+                if (k0 + j < K) {
+                    load_awaited(xv[j], reinterpret_cast<const VecT *>(plane + (int64_t)(k0 + j) * P) + i);
+                    load_awaited(dv[j], reinterpret_cast<const VecT *>(isd + (int64_t)(k0 + j) * P) + i);
                 }
-                if (d[v] <= 0.f) snr[v] = 0.f;
+#pragma unroll
+            for (int j = 0; j < KB; j++) {
+                const int k = k0 + j;
+                if (k >= K) break;
+                const float *x = reinterpret_cast<const float *>(&xv[j]);
+                const float *d = reinterpret_cast<const float *>(&dv[j]);
+                float snr[V];
+#pragma unroll
+                for (int v = 0; v < V; v++) {
+                    snr[v] = x[v] * d[v];
+                    if (d[v] > 0.f && (arg[v] < 0 || snr[v] > best[v])) {
+                        best[v] = snr[v];
+                        arg[v] = k;
+                    }
+                    if (d[v] <= 0.f) snr[v] = 0.f;
+                }
+                if (snr_all)
+                    reinterpret_cast<VecT *>(snr_all + (int64_t)k * P)[i] = *reinterpret_cast<const VecT *>(snr);
             }
-            if (snr_all) reinterpret_cast<VecT *>(snr_all + (int64_t)k * P)[i] = *reinterpret_cast<const VecT *>(snr);
         }
 #pragma unroll
         for (int v = 0; v < V; v++) {
@@ -679,7 +725,7 @@ __global__ void k_finalize_planes(const float *__restrict__ plane, const float *
 }  // namespace
 
 int fac_finalize_enqueue(const float *plane, const float *isd, int K, int64_t P, float *snr_max, int32_t *argmax,
-                         float *snr_all, const int *slot, int *global_status, void *stream, char *err,
+                         float *snr_all, const int *slot, int *global_status, bool early, void *stream, char *err,
                          size_t errlen) {
     if (P <= 0) return 0;
     // four pixels a thread once they still fill the SMs (128^2 pixels: 64 blocks
@@ -688,13 +734,9 @@ int fac_finalize_enqueue(const float *plane, const float *isd, int K, int64_t P,
     const int64_t items = vec ? P / 4 : P;
     int64_t blocks = (items + 255) / 256;
     if (blocks > 152 * 16) blocks = 152 * 16;
-    if (vec)
-        k_finalize_planes<4><<<(unsigned)blocks, 256, 0, (cudaStream_t)stream>>>(plane, isd, K, P, snr_max, argmax,
-                                                                                 snr_all, slot, global_status);
-    else
-        k_finalize_planes<1><<<(unsigned)blocks, 256, 0, (cudaStream_t)stream>>>(plane, isd, K, P, snr_max, argmax,
-                                                                                 snr_all, slot, global_status);
-    const cudaError_t e = cudaGetLastError();
+    const cudaError_t e =
+        launch_after(early, vec ? k_finalize_planes<4> : k_finalize_planes<1>, dim3((unsigned)blocks), dim3(256), 0,
+                     (cudaStream_t)stream, plane, isd, K, P, snr_max, argmax, snr_all, slot, global_status);
     if (e != cudaSuccess) {
         snprintf(err, errlen, "k_finalize_planes: %s", cudaGetErrorString(e));
         return (int)e;
@@ -773,8 +815,7 @@ int fac_enqueue(const void *tensor_map, const FacParams &p, int tw, int taps, in
         return (int)e;
     }
     if (nblocks <= 0) return 0;
-    kern<<<(unsigned)nblocks, warps * 32, smem, (cudaStream_t)stream>>>(map, p);
-    e = cudaGetLastError();
+    e = launch_after(true, kern, dim3((unsigned)nblocks), dim3(warps * 32), smem, (cudaStream_t)stream, map, p);
     if (e != cudaSuccess) {
         snprintf(err, errlen, "k_numerator_fac: %s", cudaGetErrorString(e));
         return (int)e;

@@ -6,6 +6,10 @@
 #include <cstdint>
 #include <vector>
 
+#ifdef __CUDACC__
+#include <cuda_runtime.h>
+#endif
+
 #include "../../include/mf.h"
 
 namespace mf {
@@ -436,7 +440,7 @@ struct FacParams {
 // The search's status slot is copied into the device-wide status word (first
 // failure wins) by the finalisation.
 int fac_finalize_enqueue(const float *plane, const float *isd, int K, int64_t P, float *snr_max, int32_t *argmax,
-                         float *snr_all, const int *slot, int *global_status, void *stream, char *err,
+                         float *snr_all, const int *slot, int *global_status, bool early, void *stream, char *err,
                          size_t errlen);
 // CTAs of segment `seg` of a factored search: groups x tile columns x tile
 // rows ceil((H + spread) / tile_h), spread the widest of the segment's groups.
@@ -486,5 +490,25 @@ struct ProfToken {
 ProfToken prof_begin(int kid, void *stream);
 void prof_end(const ProfToken &t);
 int profile_read(mf_profile *out, int reset);
+
+#ifdef __CUDACC__
+// Launch `kern`; `early`: as a programmatic dependent of the kernel before it in
+// the stream, so that it may start while that one's last CTAs run, and orders
+// itself with wait_previous().
+template <typename... KA, typename... A>
+cudaError_t launch_after(bool early, void (*kern)(KA...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, A... args) {
+    cudaLaunchConfig_t c = {};
+    c.gridDim = grid;
+    c.blockDim = block;
+    c.dynamicSmemBytes = smem;
+    c.stream = stream;
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    c.attrs = &at;
+    c.numAttrs = early ? 1 : 0;
+    return cudaLaunchKernelEx(&c, kern, static_cast<KA>(args)...);
+}
+#endif
 
 }  // namespace mf

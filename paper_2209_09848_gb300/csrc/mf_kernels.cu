@@ -59,11 +59,16 @@ __device__ __forceinline__ float to_f32<__half>(__half v) { return __half2float(
 
 // ------------------------------------------------------------- lambda ---
 
-// Also the largest lambda, into *lmax_bits (cleared before; lambda >= 0, so
-// the float bits order as unsigned integers).
+// Also the search's status area (16 bytes): LMAX (cleared before): the largest
+// lambda, into its third word (lambda >= 0, so the float bits order as unsigned
+// integers); otherwise it is cleared here (a fill of its own would be one more
+// operation in the stream).
+template <bool LMAX>
 __global__ void k_lambda(const float *__restrict__ sigma, const uint8_t *__restrict__ mask, int64_t H,
                          int64_t W, int64_t pad, int64_t lw, int64_t lh, float *__restrict__ lam,
-                         unsigned int *lmax_bits) {
+                         unsigned int *status_area) {
+    launch_dependents();
+    if (!LMAX && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < 4) status_area[threadIdx.x] = 0u;
     float vmax = 0.f;
     for (int64_t row = blockIdx.y; row < lh; row += gridDim.y)
         for (int64_t col = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; col < lw;
@@ -79,9 +84,11 @@ __global__ void k_lambda(const float *__restrict__ sigma, const uint8_t *__restr
             lam[row * lw + col] = v;
             vmax = fmaxf(vmax, v);
         }
+    if constexpr (LMAX) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) vmax = fmaxf(vmax, __shfl_xor_sync(0xffffffffu, vmax, o));
-    if ((threadIdx.x & 31) == 0 && vmax > 0.f) atomicMax(lmax_bits, __float_as_uint(vmax));
+        for (int o = 16; o > 0; o >>= 1) vmax = fmaxf(vmax, __shfl_xor_sync(0xffffffffu, vmax, o));
+        if ((threadIdx.x & 31) == 0 && vmax > 0.f) atomicMax(status_area + 2, __float_as_uint(vmax));
+    }
 }
 
 // ------------------------------------------------------------- weight ---
@@ -140,6 +147,8 @@ __global__ void k_weight(const TIn *__restrict__ r, int64_t fstride, int64_t rst
                          TOut *__restrict__ y, int64_t T, int64_t H, int64_t W, int64_t yp,
                          const unsigned int *lmax_bits, float *__restrict__ beta) {
     constexpr bool kHalfScaled = std::is_same<TOut, __half>::value;
+    wait_previous();
+    launch_dependents();
     const float lmax = kHalfScaled ? __uint_as_float(*lmax_bits) : 0.f;
     const int64_t wq = (W + 3) / 4, rows = T * H;
     const int lane = threadIdx.x & 31;
@@ -153,29 +162,44 @@ __global__ void k_weight(const TIn *__restrict__ r, int64_t fstride, int64_t rst
         const float *lrow = lam + (yy + pad) * lw + pad;  // padded: columns W .. W + 3 exist
         const TIn *rrow = r + t * fstride + yy * rstride;
         TOut *yrow = y + ri * yp;
-        for (int64_t xq = lane; xq < wq; xq += 32) {
-            const int64_t x0 = xq * 4;
-            const float4 l4 = *reinterpret_cast<const float4 *>(lrow + x0);
-            const float l[4] = {l4.x, l4.y, l4.z, l4.w};
-            float v[4];
-            if (VR && x0 + 4 <= W) {
-                load4_f32(rrow + x0, v);
-            } else {
+        // two chunks of four pixels a lane, their loads before their stores (1000
+        // x 2048^2 frames: 5.42 ms, one after the other 5.85, four chunks 5.36;
+        // 600 x 512^2 bf16: 0.17 ms, four chunks 0.20)
+        constexpr int NC = 2;
+        for (int64_t xb = lane; xb < wq; xb += 32 * NC) {
+            float4 l4[NC] = {};
+            float v[NC][4] = {};
 #pragma unroll
-                for (int j = 0; j < 4; j++) v[j] = x0 + j < W ? to_f32(rrow[x0 + j]) : 0.f;
-            }
-            float o[4];
+            for (int c = 0; c < NC; c++) {
+                const int64_t x0 = (xb + 32 * c) * 4;
+                if (x0 >= W) continue;
+                load_awaited(l4[c], reinterpret_cast<const float4 *>(lrow + x0));
+                if (VR && x0 + 4 <= W) {
+                    load4_f32(rrow + x0, v[c]);
+                } else {
 #pragma unroll
-            for (int j = 0; j < 4; j++) {
-                o[j] = (x0 + j < W) ? l[j] * (sc * v[j]) : 0.f;
-                if (kHalfScaled) o[j] *= inv;  // a power of two: exact
+                    for (int j = 0; j < 4; j++) v[c][j] = x0 + j < W ? to_f32(rrow[x0 + j]) : 0.f;
+                }
             }
-            TOut *dst = yrow + x0;
-            if (std::is_same<TOut, float>::value) {
-                *reinterpret_cast<float4 *>(dst) = make_float4(o[0], o[1], o[2], o[3]);
-            } else {
-                TOut q[4] = {from_f32<TOut>(o[0]), from_f32<TOut>(o[1]), from_f32<TOut>(o[2]), from_f32<TOut>(o[3])};
-                *reinterpret_cast<uint2 *>(dst) = *reinterpret_cast<const uint2 *>(q);
+#pragma unroll
+            for (int c = 0; c < NC; c++) {
+                const int64_t x0 = (xb + 32 * c) * 4;
+                if (x0 >= W) continue;
+                const float l[4] = {l4[c].x, l4[c].y, l4[c].z, l4[c].w};
+                float o[4];
+#pragma unroll
+                for (int j = 0; j < 4; j++) {
+                    o[j] = (x0 + j < W) ? l[j] * (sc * v[c][j]) : 0.f;
+                    if (kHalfScaled) o[j] *= inv;  // a power of two: exact
+                }
+                TOut *dst = yrow + x0;
+                if (std::is_same<TOut, float>::value) {
+                    *reinterpret_cast<float4 *>(dst) = make_float4(o[0], o[1], o[2], o[3]);
+                } else {
+                    TOut q[4] = {from_f32<TOut>(o[0]), from_f32<TOut>(o[1]), from_f32<TOut>(o[2]),
+                                 from_f32<TOut>(o[3])};
+                    *reinterpret_cast<uint2 *>(dst) = *reinterpret_cast<const uint2 *>(q);
+                }
             }
         }
     }
@@ -388,6 +412,10 @@ __global__ void __launch_bounds__(32 * C / NO, 256 / C) k_den_box(
                 if (px + c < W) dst[c] = o[c];
         }
     }
+    // started early, it ends after the kernel before it: what follows may read
+    // what both wrote
+    launch_dependents();
+    if (blockIdx.x == 0 && blockIdx.y == 0) wait_previous();
 }
 
 // ---------------------------------------------------------- numerator ---
@@ -903,37 +931,43 @@ int den_tile_cols(const mf_prf_table &tab, int64_t W) {
     return best;
 }
 
-// Inverse variance, weighted stack, denominator and (general numerator) a
-// cleared key buffer.
-int enqueue_pre(const SearchArgs &a, cudaStream_t stream, char *err, size_t errlen) {
+// Inverse variance and weighted stack; `early`: the second as a programmatic
+// dependent of the first (not in a batch, whose side streams fill the device
+// already: its waiting CTAs would take the other searches' places).
+int enqueue_pre(const SearchArgs &a, bool early, cudaStream_t stream, char *err, size_t errlen) {
     const mf_stack &st = *a.stack;
-    const mf_prf_table &tab = *a.tab;
     const WorkspaceLayout &L = a.L;
-    const int64_t T = st.T, H = st.H, W = st.W, P = H * W;
+    const int64_t T = st.T, H = st.H, W = st.W;
     float *lam = reinterpret_cast<float *>(a.ws + L.lam_off);
     void *y = a.ws + L.y_off;
     float *beta = reinterpret_cast<float *>(a.ws + L.beta_off);
-    float *isd = reinterpret_cast<float *>(a.ws + L.isd_off);
-    unsigned long long *keys = reinterpret_cast<unsigned long long *>(a.ws + L.keys_off);
     unsigned int *lmax = reinterpret_cast<unsigned int *>(a.ws + L.status_off + 8);
     // the search's status slot and the lambda maximum start clear (the
-    // kernels after this in stream order write the slot only on a failure)
-    cudaError_t e0 = cudaMemsetAsync(a.ws + L.status_off, 0, 16, stream);
-    if (e0 != cudaSuccess) {
-        snprintf(err, errlen, "cudaMemsetAsync: %s", cudaGetErrorString(e0));
-        return (int)e0;
+    // kernels after this in stream order write the slot only on a failure);
+    // only fp16 weighted stacks need the maximum
+    unsigned int *area = reinterpret_cast<unsigned int *>(a.ws + L.status_off);
+    const bool need_max = st.dtype == MF_F16 && L.ybytes == 2;
+    if (need_max) {
+        const cudaError_t e0 = cudaMemsetAsync(area, 0, 16, stream);
+        if (e0 != cudaSuccess) {
+            snprintf(err, errlen, "cudaMemsetAsync: %s", cudaGetErrorString(e0));
+            return (int)e0;
+        }
     }
     {
         LaunchScope ls(kKLambda, stream);
         // rows and columns by grid dimension (no 64-bit division per pixel); a
-        // few blocks per SM, since every warp ends in an atomic maximum
-        const int64_t gx = (L.lam_w + 127) / 128, gy = std::max<int64_t>(1, std::min(L.lam_h, 152 * 16 / gx));
+        // few blocks per SM, since with the maximum every warp ends in an atomic
+        // (2048^2: 78 us with 32 per SM, 88 with 16)
+        const int64_t gx = (L.lam_w + 127) / 128, gy = std::max<int64_t>(1, std::min(L.lam_h, 152 * 32 / gx));
         const dim3 grid((unsigned)std::min<int64_t>(gx, 65535), (unsigned)gy);
-        k_lambda<<<grid, 128, 0, stream>>>(a.sigma, a.mask, H, W, L.pad, L.lam_w, L.lam_h, lam, lmax);
+        (need_max ? k_lambda<true> : k_lambda<false>)<<<grid, 128, 0, stream>>>(a.sigma, a.mask, H, W, L.pad, L.lam_w,
+                                                                               L.lam_h, lam, area);
     }
     MF_CHECK_LAUNCH("k_lambda");
 
     const int64_t fs = st.frame_stride, rs = st.row_stride;
+    cudaError_t we = cudaSuccess;
     {
         LaunchScope ls(kKWeight, stream);
         const int gw = grid_for(T * H * 32, 256);  // a warp per (frame, row)
@@ -944,9 +978,9 @@ int enqueue_pre(const SearchArgs &a, cudaStream_t stream, char *err, size_t errl
         auto go = [&](auto tin, auto tout, auto vrc) {
             using TI = decltype(tin);
             using TO = decltype(tout);
-            k_weight<TI, TO, decltype(vrc)::value><<<gw, 256, 0, stream>>>(
-                (const TI *)st.data, fs, rs, st.frame_scale, lam, L.pad, L.lam_w, (TO *)y, T, H, W, L.y_pitch, lmax,
-                beta);
+            we = launch_after(early, k_weight<TI, TO, decltype(vrc)::value>, dim3(gw), dim3(256), 0, stream,
+                              (const TI *)st.data, fs, rs, st.frame_scale, (const float *)lam, L.pad, L.lam_w, (TO *)y,
+                              T, H, W, L.y_pitch, (const unsigned int *)lmax, beta);
         };
         auto go2 = [&](auto tin, auto tout) {
             if (vr) go(tin, tout, std::true_type{});
@@ -958,7 +992,28 @@ int enqueue_pre(const SearchArgs &a, cudaStream_t stream, char *err, size_t errl
         else if (y16) go2(__half{}, __half{});
         else go2(__half{}, float{});
     }
-    MF_CHECK_LAUNCH("k_weight");
+    if (we != cudaSuccess) {
+        snprintf(err, errlen, "k_weight: %s", cudaGetErrorString(we));
+        return (int)we;
+    }
+    return 0;
+}
+
+// The denominator; `early`: as a programmatic dependent of the numerator's last
+// launch.  It needs lambda only, complete since that numerator's first segment
+// waited for the weighted stack, so it takes the SMs the numerator's last CTAs
+// leave (a factored search needs 1 / sqrt(D) only at its finalisation).  With
+// that and every kernel of a factored search started early, 333 frames of 301 x
+// 277 pixels and 54 trajectories take 707 us instead of 783, 32 frames of 128 x
+// 128 and 16 trajectories 43.5 instead of 47.2; the general numerator's keys hold final SNR, so its
+// denominator comes first.  (For that numerator also a cleared key buffer.)
+int enqueue_den(const SearchArgs &a, bool early, cudaStream_t stream, char *err, size_t errlen) {
+    const mf_prf_table &tab = *a.tab;
+    const WorkspaceLayout &L = a.L;
+    const int64_t H = a.stack->H, W = a.stack->W, P = H * W;
+    const float *lam = reinterpret_cast<const float *>(a.ws + L.lam_off);
+    float *isd = reinterpret_cast<float *>(a.ws + L.isd_off);
+    unsigned long long *keys = reinterpret_cast<unsigned long long *>(a.ws + L.keys_off);
     if (tab.den_th > 0) {
         // staged: one CTA per (tile of den_th x C start pixels, trajectory)
         const int th = tab.den_th, C = den_tile_cols(tab, W);
@@ -976,9 +1031,17 @@ int enqueue_pre(const SearchArgs &a, cudaStream_t stream, char *err, size_t errl
             return (int)ea;
         }
         LaunchScope ls(kKDenominator, stream);
-        kern<<<grid, th * C / kDenOut, smem, stream>>>(lam, L.lam_w, L.lam_h, L.pad, tab.d_runs, tab.d_run_off,
-                                                       tab.d_wts, tab.d_boxes, tab.K, H, W, nbx, th, isd);
-        MF_CHECK_LAUNCH("k_den_box");
+        const dim3 block((unsigned)(th * C / kDenOut));
+        const RunRec *runs = tab.d_runs;
+        const int32_t *run_off = tab.d_run_off;
+        const float *wts = tab.d_wts;
+        const DenBox *boxes = tab.d_boxes;
+        const cudaError_t el = launch_after(early, kern, grid, block, smem, stream, lam, L.lam_w, L.lam_h, L.pad, runs,
+                                            run_off, wts, boxes, tab.K, H, W, nbx, th, isd);
+        if (el != cudaSuccess) {
+            snprintf(err, errlen, "k_den_box: %s", cudaGetErrorString(el));
+            return (int)el;
+        }
     } else {
         const int nbx = (int)((W + kDenCols - 1) / kDenCols);
         const int nby = (int)((H + 7) / 8);
@@ -1125,7 +1188,7 @@ NumBatchKernel pick_numerator_batch(int shape) {
     }
 }
 
-int enqueue_finalize(const SearchArgs &a, cudaStream_t stream, char *err, size_t errlen) {
+int enqueue_finalize(const SearchArgs &a, bool early, cudaStream_t stream, char *err, size_t errlen) {
     const int64_t P = a.stack->H * a.stack->W;
     const int *slot = reinterpret_cast<const int *>(a.ws + a.L.status_off);
     int *gstatus = status_word(err, errlen);
@@ -1134,7 +1197,7 @@ int enqueue_finalize(const SearchArgs &a, cudaStream_t stream, char *err, size_t
         LaunchScope ls(kKFinalize, stream);
         return fac_finalize_enqueue(reinterpret_cast<const float *>(a.ws + a.L.planes_off),
                                     reinterpret_cast<const float *>(a.ws + a.L.isd_off), a.tab->K, P, a.snr_max,
-                                    a.argmax, a.snr_all, slot, gstatus, stream, err, errlen);
+                                    a.argmax, a.snr_all, slot, gstatus, early, stream, err, errlen);
     }
     unsigned long long *keys = reinterpret_cast<unsigned long long *>(a.ws + a.L.keys_off);
     {
@@ -1150,8 +1213,10 @@ int enqueue_finalize(const SearchArgs &a, cudaStream_t stream, char *err, size_t
 int launch_search(const SearchArgs &a, char *err, size_t errlen) {
     cudaStream_t stream = (cudaStream_t)a.stream;
     const Plan &pl = a.tab->plan;
-    int rc = enqueue_pre(a, stream, err, errlen);
+    int rc = enqueue_pre(a, true, stream, err, errlen);
     if (rc) return rc;
+    const bool early_den = pl.kernel == 2 && a.tab->den_th > 0;
+    if (!early_den && (rc = enqueue_den(a, false, stream, err, errlen))) return rc;
     CUtensorMap map;
     if (pl.kernel == 2) {
         FacParams fp;
@@ -1168,7 +1233,8 @@ int launch_search(const SearchArgs &a, char *err, size_t errlen) {
                              stream, err, errlen);
             if (rc) return rc;
         }
-        return enqueue_finalize(a, stream, err, errlen);
+        if (early_den && (rc = enqueue_den(a, true, stream, err, errlen))) return rc;
+        return enqueue_finalize(a, true, stream, err, errlen);
     }
     NumParams np;
     int tiles_y = 0;
@@ -1187,7 +1253,7 @@ int launch_search(const SearchArgs &a, char *err, size_t errlen) {
         kern<<<(unsigned)nblocks, kWarps * 32, smem, stream>>>(map, np);
         MF_CHECK_LAUNCH("k_numerator");
     }
-    return enqueue_finalize(a, stream, err, errlen);
+    return enqueue_finalize(a, true, stream, err, errlen);
 }
 
 // ------------------------------------------------------------ batching ---
@@ -1401,7 +1467,8 @@ int batch_enqueue(BatchDevice *b, const SearchArgs *items, int n, void *stream_v
         return (int)e;
     }
     for (int i = 0; i < n; i++) {
-        int rc = enqueue_pre(items[i], b->side[i % BatchDevice::kSide], err, errlen);
+        int rc = enqueue_pre(items[i], false, b->side[i % BatchDevice::kSide], err, errlen);
+        if (!rc) rc = enqueue_den(items[i], false, b->side[i % BatchDevice::kSide], err, errlen);
         if (rc) return rc;
     }
     for (int s = 0; s < BatchDevice::kSide && e == cudaSuccess; s++) {
@@ -1448,7 +1515,7 @@ int batch_enqueue(BatchDevice *b, const SearchArgs *items, int n, void *stream_v
         if (rc) return rc;
     }
     for (int i = 0; i < n; i++) {
-        int rc = enqueue_finalize(items[i], lane(b->item_chain[i]), err, errlen);
+        int rc = enqueue_finalize(items[i], false, lane(b->item_chain[i]), err, errlen);
         if (rc) return rc;
     }
     for (int s = 0; s < BatchDevice::kSide && e == cudaSuccess; s++) {

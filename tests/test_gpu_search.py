@@ -472,3 +472,47 @@ def test_small_images_take_shorter_tiles(mf, oracle, H, W, layout, dtype):
         N, D = oracle.search_weighted(y16, beta, lam, sh, tp)
         smax, amax, sall = _run(mf, deq, c["sigma"], c["mask"], table, dtype=torch.bfloat16)
     check_search(smax, amax, sall, N, D, oracle, label="%s %s" % ((H, W), layout))
+
+
+@pytest.mark.parametrize("layout", [{}, dict(kernel=2, segments=3), dict(kernel=2, segments=1), dict(kernel=1)])
+@pytest.mark.parametrize("dtype", [torch.float32, torch.float16])
+def test_searches_back_to_back_and_captured(mf, layout, dtype):
+    # a search's kernels overlap at their ends: three different searches that
+    # share one workspace without a synchronisation between them, and the same
+    # three as a replayed graph, give what each gives alone
+    from paper_2209_09848_gb300 import synth
+    T, H, W = 48, 150, 140
+    vx, vy = synth.velocity_grid(3, 3, -0.4, 0.4)
+    table = mf.prf_table_create(vx, vy, T, **layout)
+    cs = [synth.small_case(T, H, W, seed, mask_frac=0.02, movers=2) for seed in (5, 6, 7)]
+    args = [(torch.from_numpy(c["res"]).cuda().to(dtype), torch.from_numpy(c["sigma"] * (1.0 + i)).cuda().float(),
+             torch.from_numpy(c["mask"]).cuda()) for i, c in enumerate(cs)]
+    outs = [(torch.zeros((H, W), device="cuda"), torch.zeros((H, W), dtype=torch.int32, device="cuda"),
+             torch.zeros((9, H, W), device="cuda")) for _ in cs]
+    ws = torch.empty(mf.search_workspace_size((T, H, W), table, dtype), dtype=torch.uint8, device="cuda")
+    alone = []
+    for r, s, m in args:
+        alone.append([x.clone() for x in mf.search(r, s, table, mask=m, want_all=True)])
+        torch.cuda.synchronize()
+
+    def all_three():
+        for (r, s, m), o in zip(args, outs):
+            mf.search(r, s, table, mask=m, workspace=ws, out=o)
+
+    def same():
+        torch.cuda.synchronize()
+        for o, a in zip(outs, alone):
+            for x, y in zip(o, a):
+                assert torch.equal(x, y)
+                x.zero_()
+
+    for _ in range(5):
+        all_three()
+    same()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        all_three()
+    for _ in range(5):
+        graph.replay()
+    same()
+    assert mf.device_status() == 0
