@@ -11,7 +11,7 @@
 //                  stores 1 / sqrt(D);
 //   k_numerator    N_k(p) = sum_t sum_ab W y_t, the gather stencil: frame
 //                  windows staged in shared memory by TMA and reused by the
-//                  eight trajectories of a CTA, 25 FP32 FMAs per
+//                  2 to 16 trajectories of a CTA, 25 FP32 FMAs per
 //                  (trajectory, pixel, frame); epilogue forms SNR, reduces the
 //                  max / argmax over the CTA's trajectories and merges it into
 //                  a per-pixel 64-bit key with atomicMax;
@@ -503,7 +503,8 @@ __device__ __forceinline__ void stencil_dispatch(const float *__restrict__ base,
 }
 
 // One CTA: an output tile of (32 TYS) x (32 TXS) start pixels for KT
-// trajectories, kWarps warps, one (trajectory, sub-tile) pair per warp.
+// trajectories, one (trajectory, sub-tile) pair per warp, kWarps warps or half
+// of them (see numerator_halves).
 // The work of one CTA on one (output tile, trajectory group): returns false
 // if it gave up (a bounded wait ran out; the device status word says why).
 // `smem` is the CTA's 1024-aligned dynamic shared memory, derived from the
@@ -511,7 +512,8 @@ __device__ __forceinline__ void stencil_dispatch(const float *__restrict__ base,
 template <int KT, int TXS, int TYS, int VEC>
 __device__ __forceinline__ bool numerator_tile(const CUtensorMap *ymap, const NumParams &p, int g, int tile,
                                                unsigned char *smem) {
-    static_assert(KT * TXS * TYS == kWarps, "one warp per (trajectory, sub-tile)");
+    constexpr int NW = KT * TXS * TYS;
+    static_assert(NW == kWarps || NW == kWarps / 2, "one warp per (trajectory, sub-tile)");
     constexpr int NS = kStages;
     constexpr int TH = kTile * TYS, TW = kTile * TXS;
     constexpr uint32_t kBlockBytes = (uint32_t)(sizeof(FrameHdr) + KT * sizeof(SlotRec));
@@ -646,7 +648,7 @@ __device__ __forceinline__ bool numerator_tile(const CUtensorMap *ymap, const Nu
         if (lane == 0) {
             __threadfence_block();
             const int prev = atomicAdd(&cnt[s], 1);
-            if (prev == kWarps - 1) {
+            if (prev == NW - 1) {
                 cnt[s] = 0;
                 if (t + NS < p.T) {
                     const FrameHdr h = *reinterpret_cast<const FrameHdr *>(fblk);
@@ -709,8 +711,8 @@ __device__ __forceinline__ bool numerator_tile(const CUtensorMap *ymap, const Nu
 }
 
 template <int KT, int TXS, int TYS, int VEC>
-__global__ void __launch_bounds__(kWarps * 32, 1) k_numerator(const __grid_constant__ CUtensorMap ymap,
-                                                              const NumParams p) {
+__global__ void __launch_bounds__(KT * TXS * TYS * 32, kWarps / (KT * TXS * TYS))
+    k_numerator(const __grid_constant__ CUtensorMap ymap, const NumParams p) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char *smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
     numerator_tile<KT, TXS, TYS, VEC>(&ymap, p, (int)(blockIdx.x % (unsigned)p.G),
@@ -1064,8 +1066,50 @@ int enqueue_den(const SearchArgs &a, bool early, cudaStream_t stream, char *err,
 }
 
 // Tensor map over the weighted stack and the numerator's parameters.
-int numerator_params(const SearchArgs &a, CUtensorMap *map, NumParams *np, int *tiles_y, char *err,
-                     size_t errlen) {
+// Tile and staged window of the general numerator's CTAs.
+struct NumGeometry {
+    int tw, th, S, BH;
+};
+
+// The plan's, or (half) the same groups on tiles of half the sub-tiles: a window
+// shrinks with its tile, which is a whole number of 32-column sub-tiles or of
+// 32 rows smaller.
+NumGeometry numerator_geometry(const Plan &pl, bool half) {
+    NumGeometry g = {pl.tile_w(), pl.tile_h(), pl.S, pl.BH};
+    if (half) {
+        const int cut = kShapes[pl.shape].txs == kShapes[pl.shape].tys ? g.th / 2 : 0;  // 2 x 2: 2 x 1
+        if (cut) {
+            g.th -= cut;
+            g.BH -= cut;
+        } else {
+            g.S -= g.tw / 2;
+            g.tw /= 2;
+        }
+    }
+    return g;
+}
+
+long long numerator_ctas(const Plan &pl, const NumGeometry &g, int64_t H, int64_t W) {
+    return (long long)pl.G * ((W - kTileOriginX + g.tw - 1) / g.tw) * ((H + g.th - 1) / g.th);
+}
+
+// Two CTAs of 8 warps on an SM instead of one of 16: they wait for their frames
+// apart and fill the last wave better, and every sum is the same.  60 frames x 24
+// trajectories (groups of 8): 128^2 153 -> 92 us, 500 x 421 450 -> 384, 1024^2
+// 1653 -> 1555, 2048^2 6258 -> 6025; 300 x 1000^2 x 4 (groups of 2) 2783 -> 1621.
+// Not where all CTAs of 16 warps run at once and those of 8 would not, one to an
+// SM: the same two halves on the fullest SM with more halo to load (256^2: 154
+// and 156 us); nor where two windows do not fit on an SM.
+bool numerator_halves(const Plan &pl, int64_t H, int64_t W) {
+    if (kShapes[pl.shape].txs * kShapes[pl.shape].tys < 2) return false;
+    const NumGeometry g = numerator_geometry(pl, true);
+    if (numerator_smem_bytes(g.S, g.BH, pl.kt()) > (size_t)kSmemBudget / 2) return false;
+    const long long full = numerator_ctas(pl, numerator_geometry(pl, false), H, W);
+    return full > 152 || numerator_ctas(pl, g, H, W) <= 152;
+}
+
+int numerator_params(const SearchArgs &a, const NumGeometry &geo, CUtensorMap *map, NumParams *np, int *tiles_y,
+                     char *err, size_t errlen) {
     const mf_stack &st = *a.stack;
     const mf_prf_table &tab = *a.tab;
     const Plan &pl = tab.plan;
@@ -1076,7 +1120,7 @@ int numerator_params(const SearchArgs &a, CUtensorMap *map, NumParams *np, int *
     float *y = reinterpret_cast<float *>(a.ws + L.y_off);
     cuuint64_t dims[3] = {(cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)T};
     cuuint64_t strides[2] = {(cuuint64_t)L.y_pitch * 4, (cuuint64_t)(H * L.y_pitch * 4)};
-    cuuint32_t box[3] = {(cuuint32_t)pl.S, (cuuint32_t)pl.BH, 1};
+    cuuint32_t box[3] = {(cuuint32_t)geo.S, (cuuint32_t)geo.BH, 1};
     cuuint32_t estr[3] = {1, 1, 1};
     CUresult cr = g_encode(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, y, dims, strides, box, estr,
                            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
@@ -1095,11 +1139,11 @@ int numerator_params(const SearchArgs &a, CUtensorMap *map, NumParams *np, int *
     np->G = pl.G;
     np->H = H;
     np->W = W;
-    np->tiles_x = (int)((W - kTileOriginX + pl.tile_w() - 1) / pl.tile_w());
-    np->S = pl.S;
-    np->BH = pl.BH;
+    np->tiles_x = (int)((W - kTileOriginX + geo.tw - 1) / geo.tw);
+    np->S = geo.S;
+    np->BH = geo.BH;
     np->lockstep = pl.lockstep;
-    *tiles_y = (int)((H + pl.tile_h() - 1) / pl.tile_h());
+    *tiles_y = (int)((H + geo.th - 1) / geo.th);
     return 0;
 }
 
@@ -1161,9 +1205,12 @@ int fac_params(const SearchArgs &a, int th, CUtensorMap *map, FacParams *fp, cha
 typedef void (*NumKernel)(const CUtensorMap, const NumParams);
 typedef void (*NumBatchKernel)(const CUtensorMap *, const BatchItem *, int, long long, unsigned long long *);
 
-NumKernel pick_numerator(int shape, int vec) {
+NumKernel pick_numerator(int shape, int vec, bool half) {
 #define MF_PICK(V)                                       \
-    switch (shape) {                                     \
+    switch (shape + (half ? kNumShapes : 0)) {           \
+        case kNumShapes + 1: return k_numerator<8, 1, 1, V>; \
+        case kNumShapes + 2: return k_numerator<4, 2, 1, V>; \
+        case kNumShapes + 3: return k_numerator<2, 2, 2, V>; \
         case 0: return k_numerator<16, 1, 1, V>;         \
         case 1: return k_numerator<8, 2, 1, V>;          \
         case 2: return k_numerator<4, 2, 2, V>;          \
@@ -1216,7 +1263,7 @@ int launch_search(const SearchArgs &a, char *err, size_t errlen) {
     int rc = enqueue_pre(a, true, stream, err, errlen);
     if (rc) return rc;
     const bool early_den = pl.kernel == 2 && a.tab->den_th > 0;
-    if (!early_den && (rc = enqueue_den(a, false, stream, err, errlen))) return rc;
+    if (!early_den && (rc = enqueue_den(a, true, stream, err, errlen))) return rc;
     CUtensorMap map;
     if (pl.kernel == 2) {
         FacParams fp;
@@ -1238,19 +1285,21 @@ int launch_search(const SearchArgs &a, char *err, size_t errlen) {
     }
     NumParams np;
     int tiles_y = 0;
-    rc = numerator_params(a, &map, &np, &tiles_y, err, errlen);
+    const bool half = numerator_halves(pl, a.stack->H, a.stack->W);
+    const NumGeometry geo = numerator_geometry(pl, half);
+    rc = numerator_params(a, geo, &map, &np, &tiles_y, err, errlen);
     if (rc) return rc;
     {
-        const size_t smem = numerator_smem_bytes(pl.S, pl.BH, pl.kt());
-        NumKernel kern = pick_numerator(pl.shape, pl.vec);
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        const size_t smem = numerator_smem_bytes(geo.S, geo.BH, pl.kt());
+        NumKernel kern = pick_numerator(pl.shape, pl.vec, half);
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemAllow);
         if (e != cudaSuccess) {
             snprintf(err, errlen, "cudaFuncSetAttribute(smem=%zu): %s", smem, cudaGetErrorString(e));
             return (int)e;
         }
-        const long long nblocks = (long long)pl.G * np.tiles_x * tiles_y;
+        const long long nblocks = numerator_ctas(pl, geo, a.stack->H, a.stack->W);
         LaunchScope ls(kKNumerator, stream);
-        kern<<<(unsigned)nblocks, kWarps * 32, smem, stream>>>(map, np);
+        kern<<<(unsigned)nblocks, (half ? kWarps / 2 : kWarps) * 32, smem, stream>>>(map, np);
         MF_CHECK_LAUNCH("k_numerator");
     }
     return enqueue_finalize(a, true, stream, err, errlen);
@@ -1331,7 +1380,7 @@ int batch_build(const SearchArgs *items, int n, BatchDevice **out, char *err, si
             CUtensorMap m;
             BatchItem bi;
             std::memset(&bi, 0, sizeof bi);
-            int rc = numerator_params(items[i], &m, &bi.p, &bi.tiles_y, err, errlen);
+            int rc = numerator_params(items[i], numerator_geometry(items[i].tab->plan, false), &m, &bi.p, &bi.tiles_y, err, errlen);
             if (rc) {
                 batch_free(b);
                 return rc;

@@ -516,3 +516,22 @@ def test_searches_back_to_back_and_captured(mf, layout, dtype):
         graph.replay()
     same()
     assert mf.device_status() == 0
+
+
+@pytest.mark.parametrize("shape,H,W,vmax", [
+    (1, 31, 57, 0.25), (1, 32, 25, 0.25),  # one tile of either width
+    (1, 256, 256, 0.3),                    # all whole CTAs at once, not all halves
+    (2, 129, 65, 0.25), (3, 257, 130, 0.25),
+    (2, 130, 140, 1.5),                    # wide windows
+])
+def test_general_numerator_half_tiles(mf, oracle, shape, H, W, vmax):
+    # the same layout on 16-warp and 8-warp CTAs, whichever the size takes
+    from paper_2209_09848_gb300 import synth
+    T = 24
+    c = synth.small_case(T, H, W, 70 + shape, mask_frac=0.02, movers=2)
+    vx, vy = synth.velocity_grid(4, 5, -vmax, vmax)
+    table = mf.prf_table_create(vx, vy, T, shape=shape)
+    sh, tp = oracle.trajectory_table(vx, vy, T)
+    N, D = oracle.search_full(c["res"], oracle.inverse_variance(c["sigma"], c["mask"]), sh, tp)
+    smax, amax, sall = _run(mf, c["res"], c["sigma"], c["mask"], table)
+    check_search(smax, amax, sall, N, D, oracle, label="%s %s" % (shape, (H, W)))
