@@ -47,7 +47,9 @@
 namespace mf {
 namespace {
 
+using dev::launch_dependents;
 using dev::sel_key;
+using dev::wait_previous;
 using dev::widen;
 
 constexpr int kRowTile = 2048;  // output columns per k_det_rows block at most
@@ -97,7 +99,9 @@ __device__ __forceinline__ unsigned long long ord_bits(double v) {
 // Both kernels of the stage, 2048^2 with window 255: 567 -> 236 us.
 __global__ void __launch_bounds__(128) k_det_cols(const float *__restrict__ s, const int32_t *__restrict__ am, int H,
                                                   int W, int R, int chunk, double *__restrict__ c1,
-                                                  double *__restrict__ c2, int *__restrict__ cn) {
+                                                  double *__restrict__ c2, int *__restrict__ cn, SelState *st) {
+    launch_dependents();
+    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *st = SelState{};  // the next kernel's counters
     constexpr int U = 8;  // rows whose loads are in flight together
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     if (x >= W) return;
@@ -227,11 +231,13 @@ __device__ __forceinline__ void window_stats(double s1, double s2, int n, double
 // outside the image); after the prefix scan the window [x - R, x + R] of
 // column x = x0 + t is entries t + 1 .. t + 2R + 1.
 __global__ void __launch_bounds__(kRowThreads) k_det_rows(
-    const float *__restrict__ s, const int32_t *__restrict__ am, const double *__restrict__ c1,
-    const double *__restrict__ c2, const int *__restrict__ cn, int H, int W, int R, int tile, double thr,
+    const float *__restrict__ s, const int32_t *__restrict__ am, const double *c1,
+    const double *c2, const int *cn, int H, int W, int R, int tile, double thr,
     float thr_low, int submean, float *__restrict__ z_out, double *__restrict__ zd,
     unsigned long long *__restrict__ zmax, unsigned int *__restrict__ peak, int *__restrict__ npix,
     int *__restrict__ parent, int *__restrict__ cand, SelState *st) {
+    launch_dependents();
+    wait_previous();
     extern __shared__ double sm[];
     __shared__ double wt1[kRowThreads / 32], wt2[kRowThreads / 32];
     __shared__ int wtn[kRowThreads / 32];
@@ -370,9 +376,17 @@ __device__ __forceinline__ void uf_merge(int *parent, int a, int b, int *status)
     atomicCAS(status, 0, 3);
 }
 
-// The kernels below walk the list of candidates, st->ticket of them.
-__global__ void k_det_union(int *__restrict__ parent, const int *__restrict__ cand, const SelState *st, int W,
+// The kernels below walk the list of candidates, st->ticket of them.  From the
+// column sums on, each kernel of a detection starts early (see launch_after) and
+// waits for the one before it at its top: a few microseconds of work each, so
+// that the gap between two launches would be most of their time (2048^2, window
+// 255: 311 -> 296 us; 301 x 277, window 63: 120 -> 111).  What earlier
+// kernels wrote is read through pointers that are not __restrict__ (loads of
+// const __restrict__ data need not stay behind the wait).
+__global__ void k_det_union(int *__restrict__ parent, const int *cand, const SelState *st, int W,
                             int *status) {
+    launch_dependents();
+    wait_previous();
     const unsigned int n = st->ticket;
     for (unsigned int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) {
         const int i = cand[j];
@@ -387,9 +401,11 @@ __global__ void k_det_union(int *__restrict__ parent, const int *__restrict__ ca
     }
 }
 
-__global__ void k_det_peak_z(int *parent, const int *__restrict__ cand, const SelState *st,
-                             const double *__restrict__ zd, unsigned long long *__restrict__ zmax,
+__global__ void k_det_peak_z(int *parent, const int *cand, const SelState *st,
+                             const double *zd, unsigned long long *__restrict__ zmax,
                              int *__restrict__ npix, int *status) {
+    launch_dependents();
+    wait_previous();
     const unsigned int n = st->ticket;
     for (unsigned int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) {
         const int i = cand[j];
@@ -400,9 +416,11 @@ __global__ void k_det_peak_z(int *parent, const int *__restrict__ cand, const Se
     }
 }
 
-__global__ void k_det_peak_at(const int *__restrict__ parent, const int *__restrict__ cand, const SelState *st,
-                              const double *__restrict__ zd, const unsigned long long *__restrict__ zmax,
+__global__ void k_det_peak_at(const int *parent, const int *cand, const SelState *st,
+                              const double *zd, const unsigned long long *zmax,
                               unsigned int *__restrict__ peak) {
+    launch_dependents();
+    wait_previous();
     const unsigned int n = st->ticket;
     for (unsigned int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) {
         const int i = cand[j], r = parent[i];
@@ -410,9 +428,11 @@ __global__ void k_det_peak_at(const int *__restrict__ parent, const int *__restr
     }
 }
 
-__global__ void k_det_mark(const int *__restrict__ parent, const int *__restrict__ cand, SelState *st,
-                           const double *__restrict__ zd, const unsigned int *__restrict__ peak,
+__global__ void k_det_mark(const int *parent, const int *cand, SelState *st,
+                           const double *zd, const unsigned int *peak,
                            unsigned long long *__restrict__ keys) {
+    launch_dependents();
+    wait_previous();
     const unsigned int n = st->ticket;
     const unsigned int lane = threadIdx.x & 31;
     for (unsigned int j0 = blockIdx.x * blockDim.x + (threadIdx.x & ~31u); j0 < n; j0 += gridDim.x * blockDim.x) {
@@ -433,10 +453,11 @@ __global__ void k_det_mark(const int *__restrict__ parent, const int *__restrict
 // A warp per detection; its lanes sum the peak's window again from the column
 // sums of the peak's row.
 __global__ void __launch_bounds__(256) k_det_emit(
-    const unsigned long long *__restrict__ top, const SelState *st, int max_out, const int *__restrict__ parent,
-    const float *__restrict__ s, const int32_t *__restrict__ am, const double *__restrict__ zd,
-    const double *__restrict__ c1, const double *__restrict__ c2, const int *__restrict__ cn,
-    const int *__restrict__ npix, int W, int R, mf_detection *__restrict__ out, int32_t *__restrict__ n_out) {
+    const unsigned long long *top, const SelState *st, int max_out, const int *parent,
+    const float *__restrict__ s, const int32_t *__restrict__ am, const double *zd,
+    const double *c1, const double *c2, const int *cn,
+    const int *npix, int W, int R, mf_detection *__restrict__ out, int32_t *__restrict__ n_out) {
+    wait_previous();
     const int n = max_out > 0 ? (int)st->count : 0;
     const int i = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -513,27 +534,22 @@ int launch_detect(const DetectArgs &a, char *err, size_t errlen) {
     const unsigned long long *top = reinterpret_cast<const unsigned long long *>(sws + L.sel.top_off);
     int *status = status_word(err, errlen);
     if (!status) return (int)cudaErrorUnknown;
-    cudaError_t e;
+    cudaError_t e = cudaSuccess;
 #define DET_CHECK(what)                                                          \
     do {                                                                         \
-        e = cudaGetLastError();                                                  \
+        if (e == cudaSuccess) e = cudaGetLastError();                            \
         if (e != cudaSuccess) {                                                  \
             snprintf(err, errlen, "%s: %s", what, cudaGetErrorString(e));        \
             return (int)e;                                                       \
         }                                                                        \
     } while (0)
-    e = cudaMemsetAsync(st, 0, sizeof(SelState), stream);
-    if (e != cudaSuccess) {
-        snprintf(err, errlen, "cudaMemsetAsync: %s", cudaGetErrorString(e));
-        return (int)e;
-    }
     {
         // two blocks of four warps per SM, but no chunk shorter than 8 rows
         const int nbx = (W + 127) / 128, chunks = std::max(1, 2 * 152 / nbx);
         const int chunk = std::max({8, (H + chunks - 1) / chunks, (H + 65534) / 65535});
         const dim3 grid((unsigned)nbx, (unsigned)((H + chunk - 1) / chunk));
         Scope sc(kKDetStats, stream);
-        k_det_cols<<<grid, 128, 0, stream>>>(a.snr_max, a.argmax, H, W, R, chunk, c1, c2, cn);
+        k_det_cols<<<grid, 128, 0, stream>>>(a.snr_max, a.argmax, H, W, R, chunk, c1, c2, cn, st);
     }
     DET_CHECK("k_det_cols");
     {
@@ -549,18 +565,21 @@ int launch_detect(const DetectArgs &a, char *err, size_t errlen) {
         const float thr_low = (float)std::max(-3e38, std::min(3e38, low));
         Scope sc(kKDetStats, stream);
         const unsigned grid = (unsigned)(((W + tile - 1) / tile) * (int64_t)H);
-        k_det_rows<<<grid, kRowThreads, smem, stream>>>(a.snr_max, a.argmax, c1, c2, cn, H, W, R, tile, a.threshold,
-                                                        thr_low, a.subtract_mean, a.z_out, zd, zmax, peak, npix,
-                                                        parent, cand, st);
+        e = launch_after(true, k_det_rows, dim3(grid), dim3(kRowThreads), smem, stream, a.snr_max, a.argmax, c1, c2, cn,
+                         H, W, R, tile, a.threshold, thr_low, a.subtract_mean, a.z_out, zd, zmax, peak, npix, parent,
+                         cand, st);
     }
     DET_CHECK("k_det_rows");
     {
         Scope sc(kKDetComponents, stream);
         const int g = grid_for(P, 256);
-        k_det_union<<<g, 256, 0, stream>>>(parent, cand, st, W, status);
-        k_det_peak_z<<<g, 256, 0, stream>>>(parent, cand, st, zd, zmax, npix, status);
-        k_det_peak_at<<<g, 256, 0, stream>>>(parent, cand, st, zd, zmax, peak);
-        k_det_mark<<<g, 256, 0, stream>>>(parent, cand, st, zd, peak, keys);
+        const auto next = [&](auto kern, auto... args) {
+            if (e == cudaSuccess) e = launch_after(true, kern, dim3((unsigned)g), dim3(256), 0, stream, args...);
+        };
+        next(k_det_union, parent, cand, st, W, status);
+        next(k_det_peak_z, parent, cand, st, zd, zmax, npix, status);
+        next(k_det_peak_at, parent, cand, st, zd, zmax, peak);
+        next(k_det_mark, parent, cand, st, zd, peak, keys);
     }
     DET_CHECK("k_det components");
     if (a.max_out > 0) {
@@ -570,8 +589,8 @@ int launch_detect(const DetectArgs &a, char *err, size_t errlen) {
     {
         Scope sc(kKDetEmit, stream);
         const int n = a.max_out > 0 ? a.max_out : 1;
-        k_det_emit<<<(n + 7) / 8, 256, 0, stream>>>(top, st, a.max_out, parent, a.snr_max, a.argmax, zd, c1, c2, cn,
-                                                    npix, W, R, a.out, a.n_out);
+        e = launch_after(true, k_det_emit, dim3((unsigned)(n + 7) / 8), dim3(256), 0, stream, top, st, a.max_out, parent,
+                         a.snr_max, a.argmax, zd, c1, c2, cn, npix, W, R, a.out, a.n_out);
     }
     DET_CHECK("k_det_emit");
 #undef DET_CHECK

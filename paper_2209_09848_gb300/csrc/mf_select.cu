@@ -35,7 +35,9 @@
 namespace mf {
 namespace {
 
+using dev::launch_dependents;
 using dev::sel_key;
+using dev::wait_previous;
 
 constexpr int kBins = 1 << kSelFirstBits;  // of the first histogram
 constexpr int kBinShift = 64 - kSelFirstBits;
@@ -115,6 +117,7 @@ __global__ void __launch_bounds__(kThreads) k_sel_hist(const float *__restrict__
                                                        const int32_t *__restrict__ valid, int64_t P,
                                                        unsigned int *__restrict__ hist, SelState *st,
                                                        unsigned int k_top) {
+    launch_dependents();
     extern __shared__ unsigned int bins[];
     for (int j = threadIdx.x; j < kBins; j += kThreads) bins[j] = 0u;
     __syncthreads();
@@ -153,6 +156,8 @@ __global__ void __launch_bounds__(kThreads) k_sel_hist(const float *__restrict__
 __global__ void __launch_bounds__(256) k_sel_gather(const float *__restrict__ score,
                                                     const int32_t *__restrict__ valid, int64_t P,
                                                     unsigned long long *__restrict__ list, SelState *st) {
+    launch_dependents();
+    wait_previous();
     const unsigned long long from = st->prefix;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     const int lane = threadIdx.x & 31;
@@ -183,8 +188,10 @@ __global__ void __launch_bounds__(256) k_sel_gather(const float *__restrict__ sc
 // among those that share them); 0: none, the k_top-th of the whole list is
 // wanted.
 __global__ void __cluster_dims__(kCluster) __launch_bounds__(kThreads)
-    k_sel_refine(const unsigned long long *__restrict__ list, unsigned int *hist, SelState *st, unsigned int k_top,
+    k_sel_refine(const unsigned long long *list, unsigned int *hist, SelState *st, unsigned int k_top,
                  unsigned int limit, int fixed_bits) {
+    launch_dependents();
+    wait_previous();
     namespace cg = cooperative_groups;
     cg::cluster_group cl = cg::this_cluster();
     const unsigned int n = st->list;
@@ -237,9 +244,11 @@ __global__ void __cluster_dims__(kCluster) __launch_bounds__(kThreads)
     }
 }
 
-__global__ void __launch_bounds__(256) k_sel_rank(const unsigned long long *__restrict__ list,
-                                                  const unsigned long long *__restrict__ refined, const SelState *st,
+__global__ void __launch_bounds__(256) k_sel_rank(const unsigned long long *list,
+                                                  const unsigned long long *refined, const SelState *st,
                                                   unsigned int k_top, unsigned long long *__restrict__ top) {
+    launch_dependents();
+    wait_previous();
     constexpr unsigned int kTile = 2048;  // keys staged at a time
     __shared__ __align__(16) unsigned long long tile[kTile];
     __shared__ unsigned int part[8][32];
@@ -282,10 +291,10 @@ struct Scope {
 
 #define SEL_CHECK(what)                                                   \
     do {                                                                  \
-        const cudaError_t e_ = cudaGetLastError();                        \
-        if (e_ != cudaSuccess) {                                          \
-            snprintf(err, errlen, "%s: %s", what, cudaGetErrorString(e_)); \
-            return (int)e_;                                               \
+        if (e == cudaSuccess) e = cudaGetLastError();                     \
+        if (e != cudaSuccess) {                                           \
+            snprintf(err, errlen, "%s: %s", what, cudaGetErrorString(e)); \
+            return (int)e;                                                \
         }                                                                 \
     } while (0)
 
@@ -320,16 +329,18 @@ int launch_select_list(int64_t P, int32_t k_top, int fixed_bits, char *ws, const
     SelState *st = reinterpret_cast<SelState *>(ws + L.st_off);
     unsigned long long *top = reinterpret_cast<unsigned long long *>(ws + L.top_off);
     const unsigned int limit = rank_limit(k_top);
+    cudaError_t e = cudaSuccess;
     {
         Scope sc(kKCompact, stream);
-        k_sel_refine<<<kCluster, kThreads, 0, stream>>>(list, hist, st, (unsigned)k_top, limit, fixed_bits);
+        e = launch_after(true, k_sel_refine, dim3(kCluster), dim3(kThreads), 0, stream, list, hist, st, (unsigned)k_top,
+                         limit, fixed_bits);
     }
     SEL_CHECK("k_sel_refine");
     {
         const int64_t most = P < (int64_t)limit ? P : (int64_t)limit;
         Scope sc(kKSort, stream);
-        k_sel_rank<<<(unsigned)((most + 31) / 32), 256, 0, stream>>>(
-            list, reinterpret_cast<const unsigned long long *>(hist), st, (unsigned)k_top, top);
+        e = launch_after(true, k_sel_rank, dim3((unsigned)((most + 31) / 32)), dim3(256), 0, stream, list,
+                         reinterpret_cast<const unsigned long long *>(hist), st, (unsigned)k_top, top);
     }
     SEL_CHECK("k_sel_rank");
     return 0;
@@ -365,7 +376,8 @@ int launch_select(const float *score, const int32_t *valid, int64_t P, int32_t k
     SEL_CHECK("k_sel_hist");
     {
         Scope sc(kKSelect, stream);
-        k_sel_gather<<<blocks(4 * 256, 152 * 8), 256, 0, stream>>>(score, valid, P, list, st);
+        e = launch_after(true, k_sel_gather, dim3(blocks(4 * 256, 152 * 8)), dim3(256), 0, stream, score, valid, P,
+                         list, st);
     }
     SEL_CHECK("k_sel_gather");
     return launch_select_list(P, k_top, kSelFirstBits, ws, L, stream, err, errlen);
