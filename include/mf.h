@@ -471,7 +471,7 @@ mf_status mf_detect(const float *snr_max, const int32_t *argmax, int64_t H, int6
  * psi(a) = min(max(a, -delta), delta), G = sum_t phi_t phi_t^T; the output
  * residual is r_t = y_t - phi_t . beta (the matched filter's input).  The
  * library applies G^-1 through an orthonormal basis Q = Phi R^-1 (G = R^T R,
- * built on the host in FP64); FP32 sums in blocks of 32 frames. */
+ * built on the host in FP64); FP32 sums in short blocks of frames. */
 typedef struct {
     int32_t iterations;    /* clipped steps after the least-squares start, 0..1000 */
     int32_t reserved;
@@ -529,7 +529,8 @@ mf_status mf_profile_read(mf_profile *out, int32_t reset);
  * group) work from a global counter: one launch per general CTA shape
  * present, and for the factored kernel one per time segment, tile width and
  * stack element type present, in segment order, each carrying at most 192
- * searches in its parameters), then per-search finalisation.  Each search's results equal those
+ * searches in its parameters; launches of different tile widths or element
+ * types run side by side), then per-search finalisation.  Each search's results equal those
  * of mf_search on the same inputs (same per-tile code and summation order).
  *
  * Usage: mf_batch_create; mf_batch_add per search (pointers are the caller's

@@ -10,7 +10,7 @@
 // beta = R^-1 beta_Q, but with well-scaled FP32 arithmetic.
 //
 // k_refit_resident (up to kRefitMaxResident frames): a CTA keeps the whole
-// series of its pixels in registers, so HBM sees each frame value once in and
+// series of its pixels in shared memory, so HBM sees each frame value once in and
 // each residual once out (8 bytes per pixel and frame instead of (iterations
 // + 4) x 4).  k_refit (longer series): one thread per pixel re-reads its
 // series from memory on every pass.
