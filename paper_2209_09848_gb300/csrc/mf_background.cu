@@ -124,6 +124,12 @@ __global__ void __launch_bounds__(32 * NW, kResWarps / NW) k_refit_resident(
     constexpr int STEP = VEC ? 1 : QUADS;
     float4 *vt = vs + tid;
     const float4 *qt = qs + 3 * grp;
+    // The buffer of the next exchange between the warps.  It alternates through
+    // the pixel blocks too (the step's parity would start each block with the
+    // buffer that the last step of an even number of them has just used): a
+    // warp writes a buffer again only past the barrier of the exchange in
+    // between, which every warp reaches after its reads of this one.
+    int buf = 0;
     for (int64_t blk = blockIdx.x; blk < nblk; blk += gridDim.x) {
         const int64_t p = blk * PX + first;
         const bool live[4] = {p < P, p + STEP < P, p + 2 * STEP < P, p + 3 * STEP < P};
@@ -248,18 +254,19 @@ __global__ void __launch_bounds__(32 * NW, kResWarps / NW) k_refit_resident(
                 for (int i = 0; i < 3; i++) x[i] += __shfl_xor_sync(0xffffffffu, x[i], 2);
             }
             if constexpr (NW > 1) {  // and over the warps, in order, by every warp for itself
-                float *mine = &red[step & 1][warp][quad][pos];
+                float *mine = &red[buf][warp][quad][pos];
                 if (QUADS == 4 || (lane & 2) == 0) {
 #pragma unroll
                     for (int i = 0; i < 3; i++) mine[i] = x[i];
                 }
                 __syncthreads();
 #pragma unroll
-                for (int i = 0; i < 3; i++) x[i] = red[step & 1][0][quad][pos + i];
+                for (int i = 0; i < 3; i++) x[i] = red[buf][0][quad][pos + i];
 #pragma unroll
                 for (int r = 1; r < NW; r++)
 #pragma unroll
-                    for (int i = 0; i < 3; i++) x[i] += red[step & 1][r][quad][pos + i];
+                    for (int i = 0; i < 3; i++) x[i] += red[buf][r][quad][pos + i];
+                buf ^= 1;
             }
             float *mine = reinterpret_cast<float *>(&bsh[warp][quad][0]) + pos;
             __syncwarp();  // every lane has read the previous beta

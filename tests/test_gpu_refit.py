@@ -110,3 +110,23 @@ def test_refit_series_lengths(mf, T, H, W):
     from paper_2209_09848_gb300 import synth
     c = synth.background_case(T, H, W, seed=T, n=3)
     _check(mf, c, 1.345, 4)
+
+
+@pytest.mark.parametrize("T,H,W,M", [
+    (40, 171, 171, 2),     # one warp to a CTA
+    (177, 128, 128, 2),    # two, pixel count a multiple of 4
+    (353, 101, 99, 3),     # three, an odd number of steps
+    (600, 101, 99, 4),     # four
+    (1000, 80, 80, 10),    # six
+    (1200, 53, 47, 0),     # six on 8 pixels, least squares only
+])
+def test_refit_more_pixel_blocks_than_ctas(mf, T, H, W, M):
+    # every CTA goes on to a second block of pixels, with the shared memory of
+    # the first: the buffers in which its warps exchange their sums change hands
+    # after even and odd numbers of steps; in place, the residuals of one block
+    # are written beside the reads of the next
+    from paper_2209_09848_gb300 import synth
+    c = synth.background_case(T, H, W, seed=T + M, n=4)
+    a = _check(mf, c, 1.345, M)
+    b = _check(mf, c, 1.345, M, in_place=True)
+    assert torch.equal(a[0], b[0]) and torch.equal(a[1], b[1])
