@@ -770,11 +770,11 @@ FacKernel pick_fac(int tw, int taps, int etype, bool planes) {
 
 }  // namespace
 
-int fac_batch_attr(int tw, int etype, size_t smem, char *err, size_t errlen) {
+int fac_batch_attr(int tw, int etype, char *err, size_t errlen) {
     cudaError_t e = cudaFuncSetAttribute(pick_fac_batch(tw, etype), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
+                                         kSmemAllow);
     if (e != cudaSuccess) {
-        snprintf(err, errlen, "cudaFuncSetAttribute(smem=%zu): %s", smem, cudaGetErrorString(e));
+        snprintf(err, errlen, "cudaFuncSetAttribute(smem=%d): %s", kSmemAllow, cudaGetErrorString(e));
         return (int)e;
     }
     return 0;

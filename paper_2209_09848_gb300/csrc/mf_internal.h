@@ -37,8 +37,9 @@ constexpr int kDenCols = 256;        // denominator: start pixels per warp (one 
 constexpr int kFacMaxWarps = 20;
 constexpr int kSmemBudget = 220 * 1024;  // dynamic shared memory of one CTA per SM
 // The dynamic shared memory a kernel is allowed (its attribute): one value for
-// every launch, so that threads launching it with different sizes never lower
-// each other's.
+// every launch, so that threads launching it with different sizes, and batches
+// prepared with different windows before their first runs, never lower each
+// other's.
 constexpr int kSmemAllow = 224 * 1024;
 constexpr int kSmemAllowStatic = 214 * 1024;  // the same for kernels with static arrays too
 
@@ -462,9 +463,9 @@ struct FacBatchArgs {
     int n_items;
 };
 static_assert(sizeof(FacBatchArgs) <= 32000, "within the 32 KB of kernel parameters");
-// Shared-memory limit of the persistent kernel (set once, outside capture).
+// Shared-memory allowance of the persistent kernel (outside capture).
 // etype: element type of the weighted stack, an mf_dtype (MF_F32, MF_BF16, MF_F16).
-int fac_batch_attr(int tw, int etype, size_t smem, char *err, size_t errlen);
+int fac_batch_attr(int tw, int etype, char *err, size_t errlen);
 // items: host array of n_items (1 .. kFacBatchArgItems) searches, copied
 // into the launch's parameters.
 int fac_batch_enqueue(const void *maps, const FacBatchItem *items, int n_items, long long total,

@@ -1484,25 +1484,20 @@ int batch_build(const SearchArgs *items, int n, BatchDevice **out, char *err, si
     for (const auto &grp : b->groups) {
         if (e != cudaSuccess) break;
         e = cudaFuncSetAttribute(pick_numerator_batch(grp.shape), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)grp.smem);
+                                 kSmemAllow);
     }
     if (e != cudaSuccess) {
         snprintf(err, errlen, "batch set-up: %s", cudaGetErrorString(e));
         batch_free(b);
         return (int)e;
     }
-    for (int tw : {32, 64})  // one attribute per kernel: the largest layout of that tile width and type
-        for (int et : {(int)MF_F32, (int)MF_BF16, (int)MF_F16}) {
-            size_t smem = 0;
-            for (const auto &grp : b->fac)
-                if (grp.tw == tw && grp.etype == et) smem = std::max(smem, grp.smem);
-            if (smem == 0) continue;
-            const int rc = fac_batch_attr(tw, et, smem, err, errlen);
-            if (rc) {
-                batch_free(b);
-                return rc;
-            }
+    for (const auto &grp : b->fac) {
+        const int rc = fac_batch_attr(grp.tw, grp.etype, err, errlen);
+        if (rc) {
+            batch_free(b);
+            return rc;
         }
+    }
     *out = b;
     return 0;
 }

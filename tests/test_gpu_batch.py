@@ -154,6 +154,41 @@ def test_batch_splits_launches_past_the_parameter_limit(mf):
     b.destroy()
 
 
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("large,small", [
+    (dict(kernel=2, group=5, tile_h=64, tile_w=32), dict(kernel=2, group=1, tile_h=32, tile_w=32)),
+    (dict(kernel=2, group=2, tile_h=64, tile_w=64), dict(kernel=2, group=1, tile_h=32, tile_w=64)),
+    (dict(shape=1), dict(shape=1)),
+])
+def test_batch_prepared_before_one_with_smaller_windows(mf, large, small, dtype):
+    # a batch's launches are captured in its first run; one prepared in between
+    # with smaller windows, through the same kernels, leaves them their room
+    from paper_2209_09848_gb300 import synth
+
+    def batch(T, H, W, grid, vmax, layout, seed):
+        c = synth.small_case(T, H, W, seed, movers=1)
+        table = mf.prf_table_create(*synth.velocity_grid(*grid, -vmax, vmax), T, **layout)
+        r = torch.from_numpy(c["res"]).to(dtype).cuda()
+        s = torch.from_numpy(c["sigma"]).cuda()
+        b = mf.Batch()
+        b.add(r, s, table)
+        b.prepare()
+        return b, r, s, table
+
+    first = batch(40, 90, 100, (3, 4), 0.6, large, 41)
+    second = batch(12, 70, 60, (3, 3), 0.05, small, 42)
+    assert first[3].info()["smem_bytes"] > second[3].info()["smem_bytes"]
+    for b, r, s, table in (first, second):
+        b.run()
+        torch.cuda.synchronize()
+        assert mf.device_status() == 0
+        gm, ga, _ = b.outputs[0]
+        am, aa, _ = mf.search(r, s, table)
+        torch.cuda.synchronize()
+        assert torch.equal(gm, am) and torch.equal(ga, aa)
+        b.destroy()
+
+
 def test_autotuner_picks_a_timed_layout(mf, oracle):
     """The autotuner times the factored and general layouts, caches the
     winner per bucket, and the tuned table searches correctly."""
