@@ -446,8 +446,8 @@ int fac_finalize_enqueue(const float *plane, const float *isd, int K, int64_t P,
 // CTAs of segment `seg` of a factored search: groups x tile columns x tile
 // rows ceil((H + spread) / tile_h), spread the widest of the segment's groups.
 long long fac_ctas(const mf_prf_table &tab, int64_t H, int64_t W, int seg, int th);
-// Rows of a CTA's tile for this image: the plan's, or fewer when the image
-// would leave SMs without a CTA.
+// Rows of a CTA's tile for this image: the plan's, or fewer when all its CTAs
+// run at once all the same.
 int fac_tile_rows(const mf_prf_table &tab, int64_t H, int64_t W);
 struct FacBatchItem {
     FacParams p;

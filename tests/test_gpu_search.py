@@ -535,3 +535,40 @@ def test_general_numerator_half_tiles(mf, oracle, shape, H, W, vmax):
     N, D = oracle.search_full(c["res"], oracle.inverse_variance(c["sigma"], c["mask"]), sh, tp)
     smax, amax, sall = _run(mf, c["res"], c["sigma"], c["mask"], table)
     check_search(smax, amax, sall, N, D, oracle, label="%s %s" % (shape, (H, W)))
+
+
+@pytest.mark.parametrize("T,H,W,grid,vmax,segments", [
+    (37, 40, 70, (1, 1), 0.4, 1), (37, 33, 32, (2, 2), 0.4, 1), (61, 130, 64, (2, 4), 0.1, 1),
+    (48, 97, 31, (3, 5), 0.3, 2),      # every height at once
+    (40, 200, 300, (3, 5), 0.3, 1),    # two of the heights
+    (48, 150, 157, (7, 7), 0.3, 4), (64, 300, 300, (3, 3), 1.0, 8),  # the plan's: more segments than SMs for less
+])
+def test_tile_rows_fit_the_image(mf, oracle, T, H, W, grid, vmax, segments):
+    # tiles shorter than the plan's only as long as all CTAs run at once, never
+    # against a given tile height; the same sums on every height
+    import ctypes
+    from paper_2209_09848_gb300 import synth
+    lib = ctypes.CDLL(mf.library_path())
+    rows, ctas = lib._ZN2mf13fac_tile_rowsERK12mf_prf_tablell, lib._ZN2mf8fac_ctasERK12mf_prf_tablellii
+    ctas.restype = ctypes.c_longlong
+    i64 = ctypes.c_int64
+    vx, vy = synth.velocity_grid(*grid, -vmax, vmax)
+    table = mf.prf_table_create(vx, vy, T, kernel=2, segments=segments)
+    plan = table.info()["tile_h"]
+
+    def total(th):
+        return sum(ctas(table.handle, i64(H), i64(W), j, th) for j in range(segments))
+
+    took = rows(table.handle, i64(H), i64(W))
+    assert took == min([th for th in range(32, plan + 1, 32) if total(th) <= 152], default=plan)
+    given = mf.prf_table_create(vx, vy, T, kernel=2, segments=segments, tile_h=plan)
+    assert rows(given.handle, i64(H), i64(W)) == plan
+    c = synth.small_case(T, H, W, H + W, mask_frac=0.01, movers=2)
+    a = _run(mf, c["res"], c["sigma"], c["mask"], table)
+    b = _run(mf, c["res"], c["sigma"], c["mask"], given)
+    for x, y in zip(a, b):
+        assert np.array_equal(x, y)
+    if H * W < 7000:
+        sh, tp = oracle.trajectory_table(vx, vy, T)
+        N, D = oracle.search_full(c["res"], oracle.inverse_variance(c["sigma"], c["mask"]), sh, tp)
+        check_search(*a, N, D, oracle, label="%s %s" % ((H, W), grid))
