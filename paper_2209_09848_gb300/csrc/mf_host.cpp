@@ -851,12 +851,15 @@ void denominator_layouts(mf_prf_table *t, HostLayouts &out) {
         const int r0 = run_off[k], r1 = run_off[k + 1];
         if (r1 > r0) {
             int dy0 = INT32_MAX, dy1 = INT32_MIN, x0 = INT32_MAX, x1 = INT32_MIN;
+            int64_t steps = 0;
             for (int r = r0; r < r1; r++) {
+                steps += (runs[r].nch + 3) / 4;
                 dy0 = std::min(dy0, runs[r].dy);
                 dy1 = std::max(dy1, runs[r].dy);
                 x0 = std::min(x0, runs[r].x0);
                 x1 = std::max(x1, runs[r].x0 + 4 * runs[r].nch);
             }
+            t->den_steps = std::max(t->den_steps, steps);
             b.dy0 = dy0;
             b.rows = dy1 - dy0 + 1;
             b.x0 = x0;

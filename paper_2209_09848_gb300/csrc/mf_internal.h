@@ -272,6 +272,7 @@ struct mf_prf_table {
     int den_th = 0;                      // staged denominator tile rows (0: the unstaged kernel)
     // largest G_k: box rows and columns, weights, runs (the tile's shared memory)
     int den_rows = 1, den_cols = 4, den_nw = 4, den_nr = 1;
+    int64_t den_steps = 0;               // largest G_k in pieces of up to 16 columns of a run
     int32_t *d_run_off = nullptr;        // [K + 1]
     float *d_wts = nullptr;              // run weights
     double *d_wts64 = nullptr;           // the same in FP64 (re-score)

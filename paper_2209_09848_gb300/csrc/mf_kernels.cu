@@ -1600,23 +1600,32 @@ __global__ void k_lambda64(const float *__restrict__ sigma, const uint8_t *__res
 // FP64 taps (200 consecutive bytes) and the five rows of five stack values,
 // and adds w (s r) into a sum per tap; the sums meet lambda only when the
 // trajectory's base pixel changes (a slow mover stays on a pixel for tens of
-// frames), so a frame costs one FP64 FMA.  D: lambda does not depend on the
-// frame, so D is the collapsed kernel G_k (FP64, a few hundred taps) against
-// lambda, half a warp per run of it.
+// frames), so a frame costs one FP64 FMA.  Of a trajectory that leaves the
+// image, only the frames from the first to the last that reach it are walked
+// (a check in the loop itself would put the shifts' latency before the taps':
+// 1398 us instead of 621).
+//
+// D: lambda does not depend on the frame, so D is the collapsed kernel G_k
+// (FP64, a few hundred taps) against lambda, half a warp per run of it, four
+// runs' loads in flight, only the runs whose rows lie on the image.  TAPD: D
+// from the taps, a second sum beside N's, for tables where a G_k has more
+// steps of 16 columns than the 4 T that this costs at most (footprints that
+// hardly overlap: 300 frames at 5 pixels per frame, 16384 candidates, 524 us
+// against 584; shifts that jump, whose runs are mostly gaps).
 //
 // Bound: the FP64 pipe (one warp instruction per 64 cycles and scheduler) and
-// the scattered reads.  The form with lanes over frames -- 25 taps of four FP64 operations and a
-// conversion each, for N and D, and 75 scattered reads per 32 frames --
-// measured 1490 us for 4096 candidates of 1000 frames of 1024^2; this one 530
-// (FP64 pipe 45 %, 2.3 GB of scattered 64-byte DRAM reads in that time).
-// Four frames in flight and 32 warps per SM, so that 4096 candidates run at
-// once; eight frames and 16 warps: 640 us.
-template <typename TIn>
+// the scattered reads.  4096 candidates of 1000 frames of 1024^2, whole call:
+// lanes over frames (25 taps of four FP64 operations and a conversion each for
+// N and D, 75 scattered reads per 32 frames) 2016 us, this form 621; 16384 of
+// 512^2 at 3 pixels per frame, mostly off the image: 1620 and 1004 (every frame
+// and run walked: 3361).  Four frames in flight and 32 warps per SM, so that
+// 4096 candidates run at once; eight frames and 16 warps: a fifth slower.
+template <typename TIn, bool TAPD>
 __global__ void __launch_bounds__(256, 4) k_rescore(
     const TIn *__restrict__ r, int64_t fstride, int64_t rstride, const float *__restrict__ scale,
     const double *__restrict__ lam64, const double *__restrict__ taps64, const int2 *__restrict__ shifts,
     const RunRec *__restrict__ runs, const int32_t *__restrict__ run_off, const double *__restrict__ wts64,
-    const float *__restrict__ snr_max, const int32_t *__restrict__ argmax,
+    const DenBox *__restrict__ boxes, const float *__restrict__ snr_max, const int32_t *__restrict__ argmax,
     const unsigned long long *__restrict__ keys, const SelState *st, int wpc, int T, int64_t H, int64_t W,
     mf_candidate *__restrict__ out, int32_t *__restrict__ n_out) {
     constexpr int U = 4;  // frames whose loads are in flight together
@@ -1636,10 +1645,34 @@ __global__ void __launch_bounds__(256, 4) k_rescore(
         const int Hi = (int)H, Wi = (int)W;  // at most 2^20
         const int py = (int)(idx / W), px = (int)(idx % W);
         const int b = lane / 5 - 2, a = lane % 5 - 2;
-        const int t0 = (int)((int64_t)T * part / wpc), t1 = (int)((int64_t)T * (part + 1) / wpc);
+        int t0 = (int)((int64_t)T * part / wpc), t1 = (int)((int64_t)T * (part + 1) / wpc);
         const size_t kt = (size_t)k * T;
+        // rows and columns that G_k reaches; where the image does not hold them
+        // all, only the frames from the first to the last that reach it count
+        const DenBox box = boxes[k];
+        const bool rows_in = py + box.dy0 >= 0 && py + box.dy0 + box.rows <= Hi;
+        if (!rows_in || px + box.x0 < 0 || px + box.x0 + box.cols > Wi) {
+            int first = t1, last = t0;
+            for (int t = t0; t < t1; t += 128) {
+                int2 s[4];
+#pragma unroll
+                for (int u = 0; u < 4; u++) s[u] = shifts[kt + min(t + 32 * u + lane, t1 - 1)];
+#pragma unroll
+                for (int u = 0; u < 4; u++) {
+                    const unsigned int m = __ballot_sync(0xffffffffu, t + 32 * u + lane < t1 &&
+                                                                          (unsigned)(py + s[u].y + 2) < (unsigned)(Hi + 4) &&
+                                                                          (unsigned)(px + s[u].x + 2) < (unsigned)(Wi + 4));
+                    if (m) {
+                        first = min(first, t + 32 * u + __ffs(m) - 1);
+                        last = t + 32 * u + 32 - __clz(m);
+                    }
+                }
+            }
+            t0 = first;
+            t1 = last;
+        }
         int2 base = make_int2(INT_MIN, INT_MIN);
-        double lam = 0.0, acc = 0.0;
+        double lam = 0.0, acc = 0.0, acc2 = 0.0;
         const TIn *src = r;
         bool use = false;
         for (int t = t0; t < t1; t += U) {
@@ -1663,6 +1696,10 @@ __global__ void __launch_bounds__(256, 4) k_rescore(
                 if (s[u].x != base.x || s[u].y != base.y) {  // the same for the whole warp
                     num = fma(lam, acc, num);
                     acc = 0.0;
+                    if constexpr (TAPD) {
+                        den = fma(lam, acc2, den);
+                        acc2 = 0.0;
+                    }
                     base = s[u];
                     const int qy = py + base.y + b, qx = px + base.x + a;
                     const bool in = lane < 25 && (unsigned)qy < (unsigned)Hi && (unsigned)qx < (unsigned)Wi;
@@ -1672,18 +1709,52 @@ __global__ void __launch_bounds__(256, 4) k_rescore(
                 const double x = widen(use ? v[u] : 0.f);
                 if (scale) acc = fma(w[u], (double)scale[min(t + u, t1 - 1)] * x, acc);
                 else acc = fma(w[u], x, acc);
+                if constexpr (TAPD) acc2 = fma(w[u], w[u], acc2);
             }
         }
         num = fma(lam, acc, num);
-        // D: run r of G_k by half warps
-        const int r1 = run_off[k + 1];
-        for (int q = run_off[k] + 2 * part + (lane >> 4); q < r1; q += 2 * wpc) {
-            const RunRec rr = runs[q];
-            const int y = py + rr.dy;
-            if ((unsigned)y >= (unsigned)Hi) continue;
-            for (int c = lane & 15; c < 4 * rr.nch; c += 16) {
-                const int x = px + rr.x0 + c;
-                if ((unsigned)x < (unsigned)Wi) den = fma(wts64[rr.woff + c], lam64[y * W + x], den);
+        if constexpr (TAPD) den = fma(lam, acc2, den);
+        // D: runs of G_k by half warps, the loads of four before their sums
+        if constexpr (!TAPD) {
+            constexpr int R = 4;
+            int r0 = run_off[k], r1 = run_off[k + 1];
+            if (!rows_in) {  // runs ascend in dy: the first and the end of those on the image
+                for (int end = r1; r0 < end;) {
+                    const int mid = (r0 + end) >> 1;
+                    if (py + runs[mid].dy < 0) r0 = mid + 1;
+                    else end = mid;
+                }
+                for (int from = r0; from < r1;) {
+                    const int mid = (from + r1) >> 1;
+                    if (py + runs[mid].dy < Hi) from = mid + 1;
+                    else r1 = mid;
+                }
+            }
+            const int half = lane & 15;
+            for (int q = r0 + 2 * part + (lane >> 4); q < r1; q += 2 * wpc * R) {
+                double g[R], l[R];
+                unsigned int longer = 0;  // a bit per run of more than 16 columns
+#pragma unroll
+                for (int j = 0; j < R; j++) {
+                    const int at = q + 2 * wpc * j;
+                    const RunRec rr = runs[min(at, r1 - 1)];
+                    const int y = py + rr.dy, x = px + rr.x0 + half;
+                    const bool row = at < r1;
+                    const bool in = row && half < 4 * rr.nch && (unsigned)x < (unsigned)Wi;
+                    g[j] = in ? wts64[rr.woff + half] : 0.0;
+                    l[j] = in ? lam64[y * W + x] : 0.0;
+                    longer |= (unsigned int)(row && rr.nch > 4) << j;
+                }
+#pragma unroll
+                for (int j = 0; j < R; j++) den = fma(g[j], l[j], den);
+                for (int j = 0; longer; j++, longer >>= 1) {
+                    if (!(longer & 1u)) continue;
+                    const RunRec rr = runs[q + 2 * wpc * j];
+                    for (int c = half + 16; c < 4 * rr.nch; c += 16) {
+                        const int x = px + rr.x0 + c;
+                        if ((unsigned)x < (unsigned)Wi) den = fma(wts64[rr.woff + c], lam64[(py + rr.dy) * W + x], den);
+                    }
+                }
             }
         }
 #pragma unroll
@@ -1750,9 +1821,11 @@ int launch_rescore(const RescoreArgs &a, char *err, size_t errlen) {
         LaunchScope ls(kKRescore, stream);
         auto go = [&](auto t) {
             using TI = decltype(t);
-            k_rescore<TI><<<blocks, 256, 0, stream>>>(
+            const auto kern = tab.den_steps > 4LL * tab.T ? k_rescore<TI, true> : k_rescore<TI, false>;
+            kern<<<blocks, 256, 0, stream>>>(
                 (const TI *)st.data, st.frame_stride, st.row_stride, st.frame_scale, lam64, tab.d_taps64,
-                reinterpret_cast<const int2 *>(tab.d_shifts), tab.d_runs, tab.d_run_off, tab.d_wts64, a.snr_max,
+                reinterpret_cast<const int2 *>(tab.d_shifts), tab.d_runs, tab.d_run_off, tab.d_wts64, tab.d_boxes,
+                a.snr_max,
                 a.argmax, top, sst, wpc, tab.T, H, W, a.out, a.n_out);
         };
         if (st.dtype == MF_F32) go(float{});

@@ -143,3 +143,39 @@ def test_rescore_custom_footprints_and_scales(mf, oracle, k_top, T):
     ok = D > 0
     np.testing.assert_allclose(got["snr"][ok], N[ok] / np.sqrt(D[ok]), rtol=1e-9, atol=1e-9)
     np.testing.assert_allclose(got["flux"][ok], N[ok] / D[ok], rtol=1e-9, atol=1e-9)
+
+
+@pytest.mark.parametrize("scattered", [False, True])
+@pytest.mark.parametrize("k_top,T", [(3, 301), (1500, 130), (2000, 33)])
+def test_rescore_trajectories_off_the_image(mf, oracle, k_top, T, scattered):
+    # trajectories that leave the image, return to it or never reach it (only
+    # the frames and rows between count), and with one that jumps by hundreds
+    # of pixels D from the taps instead of the collapsed kernel's rows;
+    # candidates shared by 8 to 2 warps; 1e-9: FP64 sums in other orders
+    from paper_2209_09848_gb300 import synth
+    H, W = 43, 50
+    g = np.random.default_rng(T)
+    t = np.arange(T)
+    paths = [(3.0 * t, 2.0 * t), (-0.7 * t, 0.0 * t), (90 * np.sin(t / 11.0), 5 * np.sin(t / 3.0)),
+             (0.0 * t, -70 + 0.5 * t), (0.1 * t, -0.05 * t), (0.0 * t + 200, 0.0 * t - 200)]
+    if scattered:
+        paths.append((g.integers(-400, 401, T), g.integers(-400, 401, T)))
+    sh = np.round(np.array(paths)).transpose(0, 2, 1).astype(np.int32)
+    K = len(paths)
+    tp = g.uniform(0.0, 1.0, size=(K, T, 5, 5))
+    c = synth.small_case(T, H, W, 60 + T, mask_frac=0.03, movers=1)
+    table = mf.prf_table_create_custom(sh, tp)
+    s_max, a_max = synth.score_map(H, W, seed=T, K=K, mask_frac=0.0)
+    raw, n = mf.rescore_topk(torch.from_numpy(c["res"]).cuda(), torch.from_numpy(c["sigma"]).cuda(), table,
+                             torch.from_numpy(s_max).cuda(), torch.from_numpy(a_max).cuda(), k_top,
+                             mask=torch.from_numpy(c["mask"]).cuda())
+    got = mf.decode_candidates(raw, int(n.item()))
+    want = oracle.topk_order(s_max, a_max, k_top)
+    assert np.array_equal(got["y"].astype(np.int64) * W + got["x"], want)
+    lam = oracle.inverse_variance(c["sigma"], c["mask"])
+    N, D = oracle.search_points(c["res"], lam, sh, tp, (want // W).astype(np.int32), (want % W).astype(np.int32),
+                                a_max.ravel()[want])
+    ok = D > 0
+    np.testing.assert_allclose(got["snr"][ok], N[ok] / np.sqrt(D[ok]), rtol=1e-9, atol=1e-9)
+    np.testing.assert_allclose(got["flux"][ok], N[ok] / D[ok], rtol=1e-9, atol=1e-9)
+    assert np.all(got["snr"][~ok] == 0) and np.all(got["flux"][~ok] == 0)
