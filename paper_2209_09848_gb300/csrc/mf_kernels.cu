@@ -1704,10 +1704,12 @@ __global__ void __launch_bounds__(256, 4) k_rescore(
                     const int qy = py + base.y + b, qx = px + base.x + a;
                     const bool in = lane < 25 && (unsigned)qy < (unsigned)Hi && (unsigned)qx < (unsigned)Wi;
                     lam = in ? lam64[qy * W + qx] : 0.0;
-                    use = (__double2hiint(lam) | __double2loint(lam)) != 0;  // else masked, or no usable noise value: the stack's value does not matter
+                    // else off the image, masked, or no usable noise value:
+                    // neither the stack's value nor the frame's scale matters
+                    use = (__double2hiint(lam) | __double2loint(lam)) != 0;
                 }
                 const double x = widen(use ? v[u] : 0.f);
-                if (scale) acc = fma(w[u], (double)scale[min(t + u, t1 - 1)] * x, acc);
+                if (scale) acc = fma(w[u], use ? (double)scale[min(t + u, t1 - 1)] * x : 0.0, acc);
                 else acc = fma(w[u], x, acc);
                 if constexpr (TAPD) acc2 = fma(w[u], w[u], acc2);
             }

@@ -179,3 +179,37 @@ def test_rescore_trajectories_off_the_image(mf, oracle, k_top, T, scattered):
     np.testing.assert_allclose(got["snr"][ok], N[ok] / np.sqrt(D[ok]), rtol=1e-9, atol=1e-9)
     np.testing.assert_allclose(got["flux"][ok], N[ok] / D[ok], rtol=1e-9, atol=1e-9)
     assert np.all(got["snr"][~ok] == 0) and np.all(got["flux"][~ok] == 0)
+
+
+def test_rescore_ignores_scales_of_frames_without_a_pixel(mf, oracle):
+    # a frame whose footprint lies off the image or on masked pixels adds
+    # nothing, whatever its scale
+    from paper_2209_09848_gb300 import synth
+    T, H, W = 21, 40, 60
+    c = synth.small_case(T, H, W, 77, movers=1)
+    mask = np.zeros((H, W), np.uint8)
+    mask[20:34, 30:44] = 1
+    sh = np.zeros((2, T, 2), np.int32)
+    sh[:, 3] = (500, 0)
+    sh[:, 9] = (0, -300)
+    sh[:, 14] = (30, 20)  # from rows 4 .. 9, columns 4 .. 9 onto the mask
+    g = np.random.default_rng(3)
+    tp = g.uniform(0.1, 1.0, size=(2, T, 5, 5))
+    scale = g.uniform(0.5, 2.0, T).astype(np.float32)
+    bad = scale.copy()
+    bad[[3, 9, 14]] = np.inf, np.nan, -np.inf
+    a_max = np.full((H, W), -1, np.int32)
+    a_max[4:10, 4:10] = g.integers(0, 2, (6, 6))
+    s_max = g.normal(size=(H, W)).astype(np.float32)
+    table = mf.prf_table_create_custom(sh, tp)
+    raw, n = mf.rescore_topk(torch.from_numpy(c["res"]).cuda(), torch.from_numpy(c["sigma"]).cuda(), table,
+                             torch.from_numpy(s_max).cuda(), torch.from_numpy(a_max).cuda(), 30,
+                             mask=torch.from_numpy(mask).cuda(), frame_scale=torch.from_numpy(bad).cuda())
+    got = mf.decode_candidates(raw, int(n.item()))
+    want = oracle.topk_order(s_max, a_max, 30)
+    N, D = oracle.search_points(c["res"], oracle.inverse_variance(c["sigma"], mask), sh, tp,
+                                (want // W).astype(np.int32), (want % W).astype(np.int32), a_max.ravel()[want],
+                                frame_scale=scale.astype(np.float64))
+    assert np.all(D > 0)
+    np.testing.assert_allclose(got["snr"], N / np.sqrt(D), rtol=1e-9, atol=1e-9)
+    np.testing.assert_allclose(got["flux"], N / D, rtol=1e-9, atol=1e-9)
