@@ -84,6 +84,13 @@ DetectLayout detect_layout(int64_t P, int32_t max_out) {
     return L;
 }
 
+// Unbiased exponent of x, by bits (1024: not finite; -1023: 0 or subnormal).
+__device__ __forceinline__ int exponent(double x) { return (int)(((uint32_t)__double2hiint(x) >> 20) & 0x7FFu) - 1023; }
+
+// A sum from which more than 2^kSpoil times its size has been taken has lost
+// that many of its 53 bits; beyond this it is formed again.
+constexpr int kSpoil = 20;
+
 __device__ __forceinline__ unsigned long long ord_bits(double v) {
     const unsigned long long b = (unsigned long long)__double_as_longlong(v);
     return (b & 0x8000000000000000ull) ? ~b : (b | 0x8000000000000000ull);
@@ -97,6 +104,12 @@ __device__ __forceinline__ unsigned long long ord_bits(double v) {
 // (2048^2, window 255: 108 rows; one block per SM does fewer sums but leaves
 // the pipe idle behind the loads, 132 us).  The count goes by bit masks.
 // Both kernels of the stage, 2048^2 with window 255: 567 -> 236 us.
+//
+// A score that leaves a window leaves the rounding errors it caused behind: one
+// that is not finite, or whose square is 2^kSpoil times what remains, would
+// spoil its column down to the chunk's end.  Such a window is summed directly
+// (found by exponents, in integers: the FP64 pipe sets the pace), and an empty
+// one is exactly zero.
 __global__ void __launch_bounds__(128) k_det_cols(const float *__restrict__ s, const int32_t *__restrict__ am, int H,
                                                   int W, int R, int chunk, double *__restrict__ c1,
                                                   double *__restrict__ c2, int *__restrict__ cn, SelState *st) {
@@ -154,6 +167,7 @@ __global__ void __launch_bounds__(128) k_det_cols(const float *__restrict__ s, c
         }
         mi = fetch(y + U + R, 0, H, wi);
         mo = fetch(y + U - R - 1, 0, H, wo);
+        unsigned int spoilt = 0;  // a bit per row
 #pragma unroll
         for (int u = 0; u < U; u++) {
             const double di = widen(vi[u]), dn = widen(vo[u]);
@@ -162,11 +176,52 @@ __global__ void __launch_bounds__(128) k_det_cols(const float *__restrict__ s, c
             a1 -= dn;
             a2 = fma(-dn, dn, a2);
             an += (int)((ni >> u) & 1u) - (int)((no >> u) & 1u);
+            a1 = an == 0 ? 0.0 : a1;
+            a2 = an == 0 ? 0.0 : a2;
+            const int ev = (int)((__float_as_uint(vo[u]) >> 23) & 0xFFu);
+            spoilt |= (unsigned int)(an != 0 && ev != 0 &&
+                                     (ev == 255 || 2 * (ev - 127) - exponent(a2) > kSpoil)) << u;
             if (y + u < y1) {
                 const size_t i = (size_t)(y + u) * W + x;
                 c1[i] = a1;
                 c2[i] = a2;
                 cn[i] = an;
+            }
+        }
+        if (spoilt) {  // from the first such window on, row by row
+            auto one = [&](int q) {
+                const bool in = q >= 0 && q < H;
+                const size_t i = (size_t)(in ? q : 0) * W + x;
+                return in && am[i] >= 0 ? widen(s[i]) : 0.0;
+            };
+            for (int u = __ffs(spoilt) - 1; u < U && y + u < y1; u++) {
+                if ((spoilt >> u) & 1u) {
+                    const int lo = max(0, y + u - R), hi = min(H, y + u + R + 1);
+                    a1 = 0.0;
+                    a2 = 0.0;
+                    for (int q = lo; q < hi; q += U) {
+                        fetch(q, lo, hi, vi);
+#pragma unroll
+                        for (int j = 0; j < U; j++) {
+                            const double d = widen(vi[j]);
+                            a1 += d;
+                            a2 = fma(d, d, a2);
+                        }
+                    }
+                } else {
+                    const double di = one(y + u + R), dn = one(y + u - R - 1);
+                    a1 += di;
+                    a2 = fma(di, di, a2);
+                    a1 -= dn;
+                    a2 = fma(-dn, dn, a2);
+                }
+                const size_t i = (size_t)(y + u) * W + x;
+                if (cn[i] == 0) {
+                    a1 = 0.0;
+                    a2 = 0.0;
+                }
+                c1[i] = a1;
+                c2[i] = a2;
             }
         }
     }
@@ -186,17 +241,19 @@ __device__ __forceinline__ T block_exclusive_scan(T v, T *warp_tot) {
     if (lane == 31) warp_tot[warp] = inc;
     __syncthreads();
     if (warp == 0) {
-        T t = lane < (int)(blockDim.x >> 5) ? warp_tot[lane] : T(0);
-        T ti = t;
+        T ti = lane < (int)(blockDim.x >> 5) ? warp_tot[lane] : T(0);
 #pragma unroll
         for (int d = 1; d < 32; d <<= 1) {
             const T o = __shfl_up_sync(0xffffffffu, ti, d);
             if (lane >= d) ti += o;
         }
-        if (lane < (int)(blockDim.x >> 5)) warp_tot[lane] = ti - t;  // exclusive offsets of the warps
+        ti = __shfl_up_sync(0xffffffffu, ti, 1);
+        if (lane < (int)(blockDim.x >> 5)) warp_tot[lane] = lane ? ti : T(0);  // exclusive offsets of the warps
     }
     __syncthreads();
-    const T r = warp_tot[warp] + inc - v;
+    // the sums in front, never a sum less its last: a large value would take them along
+    const T before = __shfl_up_sync(0xffffffffu, inc, 1);
+    const T r = lane ? warp_tot[warp] + before : warp_tot[warp];
     __syncthreads();  // warp_tot may be reused
     return r;
 }
@@ -229,7 +286,9 @@ __device__ __forceinline__ void window_stats(double s1, double s2, int n, double
 // Horizontal window sums, z and the candidate flag for the columns x0 .. x0 +
 // tile - 1 of row y.  Shared entry j holds column lo + j, lo = x0 - R - 1 (0
 // outside the image); after the prefix scan the window [x - R, x + R] of
-// column x = x0 + t is entries t + 1 .. t + 2R + 1.
+// column x = x0 + t is entries t + 1 .. t + 2R + 1.  A window behind column sums
+// so large that their prefix has swallowed it, or not finite, is summed directly
+// from the column sums.
 __global__ void __launch_bounds__(kRowThreads) k_det_rows(
     const float *__restrict__ s, const int32_t *__restrict__ am, const double *c1,
     const double *c2, const int *cn, int H, int W, int R, int tile, double thr,
@@ -240,7 +299,7 @@ __global__ void __launch_bounds__(kRowThreads) k_det_rows(
     wait_previous();
     extern __shared__ double sm[];
     __shared__ double wt1[kRowThreads / 32], wt2[kRowThreads / 32];
-    __shared__ int wtn[kRowThreads / 32];
+    __shared__ int wtn[kRowThreads / 32], hi_exp[kRowThreads / 32], lo_exp[kRowThreads / 32];
     const int tiles = (W + tile - 1) / tile;
     const int y = (int)(blockIdx.x / tiles);
     const int x0 = (int)(blockIdx.x % tiles) * tile;
@@ -250,12 +309,26 @@ __global__ void __launch_bounds__(kRowThreads) k_det_rows(
     double *p2 = sm + L;
     int *pn = reinterpret_cast<int *>(sm + 2 * L);
     const size_t row = (size_t)y * W;
+    int e_hi = -1024, e_lo = 1024;  // exponents of the tile's column sums of squares, zeros left out
     for (int j = threadIdx.x; j < L; j += blockDim.x) {
         const int x = lo + j;
         const bool in = x >= 0 && x < W;
         p1[j] = in ? c1[row + x] : 0.0;
-        p2[j] = in ? c2[row + x] : 0.0;
+        const double q = in ? c2[row + x] : 0.0;
+        p2[j] = q;
         pn[j] = in ? cn[row + x] : 0;
+        const int e = exponent(q);
+        if (e > -1023) {
+            e_hi = max(e_hi, e);
+            e_lo = min(e_lo, e);
+        }
+    }
+    const int lane = threadIdx.x & 31;
+    e_hi = __reduce_max_sync(0xffffffffu, e_hi);
+    e_lo = __reduce_min_sync(0xffffffffu, e_lo);
+    if (lane == 0) {
+        hi_exp[threadIdx.x >> 5] = e_hi;
+        lo_exp[threadIdx.x >> 5] = e_lo;
     }
     __syncthreads();
     const int per = ((L + blockDim.x - 1) / blockDim.x) | 1;  // odd: neighbouring threads on other banks
@@ -279,7 +352,54 @@ __global__ void __launch_bounds__(kRowThreads) k_det_rows(
         pn[j] += on;
     }
     __syncthreads();
-    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int w = 0; w < kRowThreads / 32; w++) {
+        e_hi = max(e_hi, hi_exp[w]);
+        e_lo = min(e_lo, lo_exp[w]);
+    }
+    // Can a window sum have lost the bits that kSpoil allows?  Only if column
+    // sums differ by more than the 2^13 that a prefix of 4095 adds.  Has one?
+    // Then each thread sums the window of its first pixel directly, slides it
+    // over its others and starts again where a column that dwarfs it leaves:
+    // results do not depend on the tile.  (One spike of 1e15 in 500 x 2100,
+    // window 127: 314 us; clean maps as without the check.)
+    bool slid = false;
+    if (e_hi - e_lo > kSpoil - 13) {
+        bool lost = false;
+        for (int t = threadIdx.x; t < tile; t += blockDim.x) {
+            const double before = p2[t], upto = p2[t + 2 * R + 1];
+            lost = lost || (pn[t + 2 * R + 1] - pn[t] >= 2 &&
+                            (exponent(upto) == 1024 || exponent(before) - exponent(upto - before) > kSpoil));
+        }
+        slid = __syncthreads_or(lost);
+    }
+    if (slid) {
+        const int own = (tile + blockDim.x - 1) / blockDim.x, first = (int)threadIdx.x * own;
+        double s1 = 0.0, s2 = 0.0;
+        for (int t = first; t < min(tile, first + own) && x0 + t < W; t++) {
+            const int x = x0 + t;
+            bool direct = t == first;
+            if (!direct) {
+                const double out = x - R - 1 >= 0 ? c2[row + x - R - 1] : 0.0;
+                s1 += x + R < W ? c1[row + x + R] : 0.0;
+                s2 += x + R < W ? c2[row + x + R] : 0.0;
+                s1 -= x - R - 1 >= 0 ? c1[row + x - R - 1] : 0.0;
+                s2 -= out;
+                direct = exponent(out) > -1023 && (exponent(out) == 1024 || exponent(out) - exponent(s2) > kSpoil);
+            }
+            if (direct) {
+                s1 = 0.0;
+                s2 = 0.0;
+                for (int q = max(0, x - R); q <= min(W - 1, x + R); q++) {
+                    s1 += c1[row + q];
+                    s2 += c2[row + q];
+                }
+            }
+            p1[t] = s1;
+            p2[t] = s2;
+        }
+        __syncthreads();
+    }
     for (int t0 = threadIdx.x & ~31; t0 < tile; t0 += blockDim.x) {  // whole warps: they add to the list together
         const int t = t0 + lane, x = x0 + t;
         const bool in = t < tile && x < W;
@@ -291,8 +411,8 @@ __global__ void __launch_bounds__(kRowThreads) k_det_rows(
             float zf = 0.f;
             if (valid) {
                 const int n = pn[t + 2 * R + 1] - pn[t];
-                const double s1 = p1[t + 2 * R + 1] - p1[t];
-                const double s2 = p2[t + 2 * R + 1] - p2[t];
+                const double s1 = slid ? p1[t] : p1[t + 2 * R + 1] - p1[t];
+                const double s2 = slid ? p2[t] : p2[t + 2 * R + 1] - p2[t];
                 // u = n (s - mean) or n s, v = n^2 var: z = u / sqrt(v)
                 const float nf = (float)n;  // n < 2^24
                 const double nd = widen(nf), sd = widen(s[i]);

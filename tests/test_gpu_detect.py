@@ -210,3 +210,42 @@ def test_detect_far_scales(mf, oracle, scale):
     from paper_2209_09848_gb300 import synth
     s, a = synth.score_map(90, 333, seed=5, K=7)
     _compare(mf, oracle, s * np.float32(scale), a, 15, 3.0)
+
+
+@pytest.mark.parametrize("spike", [np.inf, np.nan, -np.inf, 1e15, -3e8])
+@pytest.mark.parametrize("H,W,window", [(40, 2100, 31), (150, 39000, 15), (700, 2300, 255)])
+def test_spoilt_scores_stay_in_their_windows(mf, H, W, window, spike):
+    # a score that is not finite, or dwarfs the others, counts in the windows
+    # that hold it and nowhere else: columns summed over long chunks of rows,
+    # prefixes over wide tiles, then a band without scores and one of zeros.
+    # FP64 windows summed directly at sampled pixels; the z map is FP32
+    from paper_2209_09848_gb300 import synth
+    s, a = synth.score_map(H, W, seed=H, K=9)
+    a[:3] = np.maximum(a[:3], 0)
+    at = [(1, 7), (2, 8), (2, W // 2), (1, W - 400)]
+    for y, x in at:
+        s[y, x] = spike
+    band = min(2 * window, H // 4)
+    a[H // 2:H // 2 + band] = -1
+    s[H // 2 + band:H // 2 + band + band // 2] = 0.0
+    z, det, found, written = _run(mf, s, a, window, 3.0)
+    g = np.random.default_rng(W)
+    R = window // 2
+    ys, xs = g.integers(0, H, 4000), g.integers(0, W, 4000)
+    near = g.integers(-R - 3, R + 4, (400, 2)) + np.array(at)[g.integers(0, len(at), 400)]
+    ys = np.concatenate([ys, np.clip(near[:, 0], 0, H - 1)])
+    xs = np.concatenate([xs, np.clip(near[:, 1], 0, W - 1)])
+    clean = 0
+    for y, x in zip(ys, xs):
+        w = np.s_[max(0, y - R):y + R + 1, max(0, x - R):x + R + 1]
+        v = s[w][a[w] >= 0].astype(np.float64)
+        want = 0.0
+        if a[y, x] >= 0 and v.size >= 2 and np.isfinite(v).all():
+            m = v.mean()
+            var = ((v - m) ** 2).mean()
+            clean += 1
+            if var > 1e-12 * (m * m + var):
+                want = (float(s[y, x]) - m) / np.sqrt(var)
+        assert abs(z[y, x] - want) <= (6e-8 + Z_TOL) * max(1.0, abs(want)), (y, x, z[y, x], want)
+    assert clean > 1000
+    assert found > 0
