@@ -37,9 +37,15 @@ size_t align256(size_t x) { return (x + 255) / 256 * 256; }
 // the G = 32 NW / QUADS owning frames g, g + G, g + 2 G ..: only that thread
 // touches its values, so the passes over the frames need no barrier.
 //
-// Values are held as v_t = y_t - y_0 (the constant is in the basis' span, so
-// the fit of v has the residuals of the fit of y, and y_0 returns in the
-// constant coefficient): all FP32 arithmetic sees noise-sized numbers.  A
+// Values are held as v_t = y_t - y0, y0 the median of three frames, or 0 where
+// that is within 2 delta of 0 (the constant is in the basis' span, so the fit of
+// v has the residuals of the fit of y, and y0 returns in the constant
+// coefficient): all FP32 arithmetic sees noise-sized numbers.  One frame alone
+// would not do: an outlier there would be every value's size.  Largest error of
+// the other frames' residuals against FP64, in sigma (y itself held, y0 = y_0,
+// and as it is): T = 600 on a background of 100 sigma 2.8e-5, 9.2e-7, 4.7e-7,
+// on none 3.9e-7, 9.0e-7, 4.2e-7; T = 1500 on none, 300 sigma off in frame 0,
+// 2.4e-7, 3.3e-5, 8.0e-7.  A
 // clipped step is, per frame, e = v - Q beta, the clip and the sums Q^T psi(e):
 // 12 FMAs per pixel, packed over pairs of frames (the basis pairs are read as
 // they lie; beta stands twice in registers), two frames by four pixels at a
@@ -118,6 +124,8 @@ __global__ void __launch_bounds__(32 * NW, kResWarps / NW) k_refit_resident(
     __syncthreads();
     const int64_t nblk = (P + PX - 1) / PX;
     const size_t nn = (size_t)n * n;
+    const float near = isfinite(delta) ? 2.f * delta : 0.f;  // an origin of the noise's size gains nothing
+    const int og = (lane / QUADS) % 3, of = og == 0 ? 0 : og == 1 ? T / 2 : T - 1;  // this lane's frame of the origin
     // pixel j of this thread: four consecutive ones for 128-bit accesses, else
     // QUADS apart (each access of a warp covers consecutive pixels)
     const int first = VEC ? 4 * quad : quad;
@@ -133,6 +141,11 @@ __global__ void __launch_bounds__(32 * NW, kResWarps / NW) k_refit_resident(
     for (int64_t blk = blockIdx.x; blk < nblk; blk += gridDim.x) {
         const int64_t p = blk * PX + first;
         const bool live[4] = {p < P, p + STEP < P, p + 2 * STEP < P, p + 3 * STEP < P};
+        // the values' origin: the median of three frames, one in each group of a
+        // warp; on its way before the series
+        float o[4];
+#pragma unroll
+        for (int j = 0; j < 4; j++) o[j] = data[(size_t)of * P + (live[j] ? p + j * STEP : 0)];
         {
             const float *src = data + (size_t)grp * P + p;
             for (int f = 0; f < 2 * np; f++, src += (size_t)G * P) {
@@ -147,14 +160,13 @@ __global__ void __launch_bounds__(32 * NW, kResWarps / NW) k_refit_resident(
                 }
             }
         }
-        // frame 0, the values' origin, and the pixels' places on the
-        // scattered-light grid; pixels of one cell share its corners
-        float y0[4], fy[4], fx[4];
+        // the pixels' places on the scattered-light grid; pixels of one cell
+        // share its corners
+        float fy[4], fx[4];
         int o00[4], di[4], dj[4];
 #pragma unroll
         for (int j = 0; j < 4; j++) {
             const int64_t pj = live[j] ? p + j * STEP : 0;
-            y0[j] = data[pj];
             const int r = (int)(pj / W), c = (int)(pj - (int64_t)r * W);
             const float u = grid_coord(r, n, H), w = grid_coord(c, n, W);
             const int i0 = (int)floorf(u), j0 = (int)floorf(w);
@@ -180,7 +192,15 @@ __global__ void __launch_bounds__(32 * NW, kResWarps / NW) k_refit_resident(
                 o[j] -= fmaf(fy[j], bot - top, top);
             }
         };
-        if (scatter) light(scatter, y0);
+        if (scatter) light(scatter + (size_t)of * nn, o);
+        float y0[4];
+#pragma unroll
+        for (int j = 0; j < 4; j++) {
+            const float u = __shfl_sync(0xffffffffu, o[j], quad), v = __shfl_sync(0xffffffffu, o[j], quad + QUADS),
+                        w = __shfl_sync(0xffffffffu, o[j], quad + 2 * QUADS);
+            y0[j] = fmaxf(fminf(u, v), fminf(fmaxf(u, v), w));
+            if (fabsf(y0[j]) <= near) y0[j] = 0.f;
+        }
         cp_async_wait();
         float2 s[6][4], nb[6][4];  // sums (even, odd frames) and -beta (twice) of the four pixels
         auto sums = [&](const float2 (&q)[6], const float2 (&e)[4]) {
@@ -197,13 +217,16 @@ __global__ void __launch_bounds__(32 * NW, kResWarps / NW) k_refit_resident(
                 q[2 * c + 1] = make_float2(a.z, a.w);
             }
         };
-        // e = v - Q beta of pair i
-        auto residual = [&](int i, const float2 (&q)[6], float2 (&e)[4]) {
+        auto values = [&](int i, float2 (&e)[4]) {
             const float4 a = vt[NT * 2 * i], b = vt[NT * (2 * i + 1)];
             e[0] = make_float2(a.x, a.y);
             e[1] = make_float2(a.z, a.w);
             e[2] = make_float2(b.x, b.y);
             e[3] = make_float2(b.z, b.w);
+        };
+        // e = v - Q beta of pair i
+        auto residual = [&](int i, const float2 (&q)[6], float2 (&e)[4]) {
+            values(i, e);
 #pragma unroll
             for (int k = 0; k < 6; k++)
 #pragma unroll
@@ -302,9 +325,19 @@ __global__ void __launch_bounds__(32 * NW, kResWarps / NW) k_refit_resident(
         if (live[0]) {
             float *dst = resid + (size_t)grp * P + p;
             for (int i = 0; i < np; i++) {
-                float2 q[6], e[4];
+                // the fit by itself first: its terms are smaller than the
+                // values, and so is what their sum's roundings leave
+                float2 q[6], e[4], m[4];
                 basis(i, q);
-                residual(i, q, e);
+                values(i, e);
+#pragma unroll
+                for (int j = 0; j < 4; j++) m[j] = __fmul2_rn(q[0], nb[0][j]);
+#pragma unroll
+                for (int k = 1; k < 6; k++)
+#pragma unroll
+                    for (int j = 0; j < 4; j++) m[j] = __ffma2_rn(q[k], nb[k][j], m[j]);
+#pragma unroll
+                for (int j = 0; j < 4; j++) e[j] = __fadd2_rn(e[j], m[j]);
 #pragma unroll
                 for (int h = 0; h < 2; h++, dst += (size_t)G * P) {
                     if (2 * i + h >= cnt) break;

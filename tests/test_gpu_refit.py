@@ -130,3 +130,27 @@ def test_refit_more_pixel_blocks_than_ctas(mf, T, H, W, M):
     a = _check(mf, c, 1.345, M)
     b = _check(mf, c, 1.345, M, in_place=True)
     assert torch.equal(a[0], b[0]) and torch.equal(a[1], b[1])
+
+
+@pytest.mark.parametrize("frame", [0, -1])
+@pytest.mark.parametrize("T,outlier", [(300, 150.0), (600, 300.0), (1500, 300.0)])
+def test_refit_outlier_in_an_end_frame(mf, T, outlier, frame):
+    # frames whose background is already gone, one of them hundreds of sigma
+    # off: the other frames' residuals are as good as without it (the bound of
+    # the other tests, for those frames' values) at every pixel whose FP64 fit
+    # has let go of it in these steps; elsewhere the fit is of the outlier's size,
+    # and the bound the other tests' own
+    from oracle import background as ob
+    H, W = 12, 20
+    g = np.random.default_rng(T)
+    jit = np.clip(np.cumsum(g.normal(0, 0.04, (T, 2)), 0), -0.15, 0.15)
+    D = g.normal(size=(T, H, W)).astype(np.float32)
+    D[frame] += np.float32(outlier)
+    R, _ = mf.background_refit(torch.from_numpy(D).cuda(), jit, 1.345, 10)
+    torch.cuda.synchronize()
+    _, Ro = ob.refit(D, jit, 1.345, 10)
+    rest = np.arange(T) != frame % T
+    gone = np.abs(D[rest] - Ro[rest]).max(axis=0) <= 1.0
+    err = np.abs(R.cpu().numpy().astype(np.float64) - Ro)[rest].max(axis=0)
+    tol = np.where(gone, 2e-6 * max(1.0, float(np.abs(D[rest]).max())), 2e-6 * float(np.abs(D).max()))
+    assert (err <= tol).all(), "residual max err / bound %.3g" % (err / tol).max()
