@@ -141,11 +141,6 @@ __global__ void __launch_bounds__(32 * NW, kResWarps / NW) k_refit_resident(
     for (int64_t blk = blockIdx.x; blk < nblk; blk += gridDim.x) {
         const int64_t p = blk * PX + first;
         const bool live[4] = {p < P, p + STEP < P, p + 2 * STEP < P, p + 3 * STEP < P};
-        // the values' origin: the median of three frames, one in each group of a
-        // warp; on its way before the series
-        float o[4];
-#pragma unroll
-        for (int j = 0; j < 4; j++) o[j] = data[(size_t)of * P + (live[j] ? p + j * STEP : 0)];
         {
             const float *src = data + (size_t)grp * P + p;
             for (int f = 0; f < 2 * np; f++, src += (size_t)G * P) {
@@ -160,6 +155,12 @@ __global__ void __launch_bounds__(32 * NW, kResWarps / NW) k_refit_resident(
                 }
             }
         }
+        // the values' origin: the median of three frames, one in each group of a
+        // warp (behind the series: in front of it 20.90 -> 21.05 ms at 1000 x
+        // 1024 x 2048)
+        float o[4];
+#pragma unroll
+        for (int j = 0; j < 4; j++) o[j] = data[(size_t)of * P + (live[j] ? p + j * STEP : 0)];
         // the pixels' places on the scattered-light grid; pixels of one cell
         // share its corners
         float fy[4], fx[4];
