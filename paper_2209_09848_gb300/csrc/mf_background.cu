@@ -20,6 +20,7 @@
 #include <cstdint>
 #include <cstdio>
 
+#include "mf_device.cuh"
 #include "mf_internal.h"
 
 namespace mf {
@@ -29,6 +30,8 @@ constexpr int kRefitThreads = 256;
 constexpr int kRefitChunk = 256;  // frames of Q staged in shared memory
 constexpr int kRefitBlock = 32;   // frames per FP32 partial sum
 constexpr int kRefitUnroll = 8;   // frames whose loads are in flight together
+
+using dev::widen;
 
 size_t align256(size_t x) { return (x + 255) / 256 * 256; }
 
@@ -105,12 +108,15 @@ __global__ void __launch_bounds__(32 * NW, kResWarps / NW) k_refit_resident(
     const float *data, int T, int H, int W, const float *__restrict__ scatter, int n, const float *__restrict__ Q,
     const double *__restrict__ Rinv, int iterations, float delta, int np, float *resid, float *__restrict__ coef) {
     constexpr int NT = 32 * NW, PX = 4 * QUADS, G = NT / QUADS;
+    constexpr int NX = QUADS == 16 ? 12 : QUADS == 8 ? 6 : 3;  // sums a lane keeps of its quad's 24
+    static_assert(QUADS == 2 || QUADS == 4 || QUADS == 8 || QUADS == 16, "the exchanges below");
     // [2 np][NT]: a thread's frame f at [f][tid] as loaded (four pixels); after
     // the first pass its pair i holds pixels 0, 1 of frames 2 i, 2 i + 1 at
     // [2 i] and pixels 2, 3 at [2 i + 1], each pixel's two values together
     extern __shared__ float4 vs[];
     float4 *qs = vs + (size_t)2 * np * NT;  // [np][G][3]: (q_k, q_k) of the pair's two frames, k = 0 .. 5
     __shared__ float red[2][NW][QUADS][24];
+    __shared__ double rsh[36];            // R^-1
     __shared__ float4 bsh[NW][QUADS][6];  // -beta of the quad's four pixels per basis vector (a copy per warp)
     const int64_t P = (int64_t)H * W;
     const int tid = threadIdx.x, quad = tid % QUADS, grp = tid / QUADS, warp = tid >> 5, lane = tid & 31;
@@ -121,11 +127,12 @@ __global__ void __launch_bounds__(32 * NW, kResWarps / NW) k_refit_resident(
 #pragma unroll
         for (int k = 0; k < 6; k++) dst[2 * k] = t < T ? Q[(size_t)t * kRefitBasisPitch + k] : 0.f;
     }
+    for (int j = tid; j < 36; j += NT) rsh[j] = Rinv[j];
     __syncthreads();
     const int64_t nblk = (P + PX - 1) / PX;
     const size_t nn = (size_t)n * n;
     const float near = isfinite(delta) ? 2.f * delta : 0.f;  // an origin of the noise's size gains nothing
-    const int og = (lane / QUADS) % 3, of = og == 0 ? 0 : og == 1 ? T / 2 : T - 1;  // this lane's frame of the origin
+    const int og = (lane / QUADS) % 3;  // this lane's frame of the origin
     // pixel j of this thread: four consecutive ones for 128-bit accesses, else
     // QUADS apart (each access of a warp covers consecutive pixels)
     const int first = VEC ? 4 * quad : quad;
@@ -158,9 +165,13 @@ __global__ void __launch_bounds__(32 * NW, kResWarps / NW) k_refit_resident(
         // the values' origin: the median of three frames, one in each group of a
         // warp (behind the series: in front of it 20.90 -> 21.05 ms at 1000 x
         // 1024 x 2048)
-        float o[4];
+        constexpr int NO = QUADS == 16 ? 3 : 1;  // frames a lane loads (a warp of two groups has none for the third)
+        const int of[3] = {NO == 3 || og == 0 ? 0 : og == 1 ? T / 2 : T - 1, T / 2, T - 1};
+        float o[NO][4];
 #pragma unroll
-        for (int j = 0; j < 4; j++) o[j] = data[(size_t)of * P + (live[j] ? p + j * STEP : 0)];
+        for (int i = 0; i < NO; i++)
+#pragma unroll
+            for (int j = 0; j < 4; j++) o[i][j] = data[(size_t)of[i] * P + (live[j] ? p + j * STEP : 0)];
         // the pixels' places on the scattered-light grid; pixels of one cell
         // share its corners
         float fy[4], fx[4];
@@ -193,12 +204,22 @@ __global__ void __launch_bounds__(32 * NW, kResWarps / NW) k_refit_resident(
                 o[j] -= fmaf(fy[j], bot - top, top);
             }
         };
-        if (scatter) light(scatter + (size_t)of * nn, o);
+        if (scatter)
+#pragma unroll
+            for (int i = 0; i < NO; i++) light(scatter + (size_t)of[i] * nn, o[i]);
         float y0[4];
 #pragma unroll
         for (int j = 0; j < 4; j++) {
-            const float u = __shfl_sync(0xffffffffu, o[j], quad), v = __shfl_sync(0xffffffffu, o[j], quad + QUADS),
-                        w = __shfl_sync(0xffffffffu, o[j], quad + 2 * QUADS);
+            float u, v, w;
+            if constexpr (NO == 3) {
+                u = o[0][j];
+                v = o[1][j];
+                w = o[2][j];
+            } else {
+                u = __shfl_sync(0xffffffffu, o[0][j], quad);
+                v = __shfl_sync(0xffffffffu, o[0][j], quad + QUADS);
+                w = __shfl_sync(0xffffffffu, o[0][j], quad + 2 * QUADS);
+            }
             y0[j] = fmaxf(fminf(u, v), fminf(fmaxf(u, v), w));
             if (fabsf(y0[j]) <= near) y0[j] = 0.f;
         }
@@ -260,9 +281,9 @@ __global__ void __launch_bounds__(32 * NW, kResWarps / NW) k_refit_resident(
             const float2 e[4] = {{v[0][0], v[1][0]}, {v[0][1], v[1][1]}, {v[0][2], v[1][2]}, {v[0][3], v[1][3]}};
             sums(q, e);
         }
-        float own[6];  // -beta of the values this lane sums
+        float own[NX];  // -beta of the values this lane sums
 #pragma unroll
-        for (int i = 0; i < 6; i++) own[i] = 0.f;
+        for (int i = 0; i < NX; i++) own[i] = 0.f;
         for (int step = 0;; step++) {
             float x[24];
 #pragma unroll
@@ -270,32 +291,34 @@ __global__ void __launch_bounds__(32 * NW, kResWarps / NW) k_refit_resident(
 #pragma unroll
                 for (int j = 0; j < 4; j++) x[4 * k + j] = s[k][j].x + s[k][j].y;
             // sums over the warp's groups: each exchange halves the values a
-            // lane keeps, the last one plain; a lane ends with 3 of its
+            // lane keeps, the last one plain; a lane ends with NX of its
             // quad's 24
-            int pos = halve<12>(x, lane, 16) + halve<6>(x, lane, 8) + halve<3>(x, lane, 4);
+            int pos = halve<12>(x, lane, 16);
+            if constexpr (QUADS <= 8) pos += halve<6>(x, lane, 8);
+            if constexpr (QUADS <= 4) pos += halve<3>(x, lane, 4);
             if constexpr (QUADS == 2) {
 #pragma unroll
-                for (int i = 0; i < 3; i++) x[i] += __shfl_xor_sync(0xffffffffu, x[i], 2);
+                for (int i = 0; i < NX; i++) x[i] += __shfl_xor_sync(0xffffffffu, x[i], 2);
             }
             if constexpr (NW > 1) {  // and over the warps, in order, by every warp for itself
                 float *mine = &red[buf][warp][quad][pos];
-                if (QUADS == 4 || (lane & 2) == 0) {
+                if (QUADS != 2 || (lane & 2) == 0) {
 #pragma unroll
-                    for (int i = 0; i < 3; i++) mine[i] = x[i];
+                    for (int i = 0; i < NX; i++) mine[i] = x[i];
                 }
                 __syncthreads();
 #pragma unroll
-                for (int i = 0; i < 3; i++) x[i] = red[buf][0][quad][pos + i];
+                for (int i = 0; i < NX; i++) x[i] = red[buf][0][quad][pos + i];
 #pragma unroll
                 for (int r = 1; r < NW; r++)
 #pragma unroll
-                    for (int i = 0; i < 3; i++) x[i] += red[buf][r][quad][pos + i];
+                    for (int i = 0; i < NX; i++) x[i] += red[buf][r][quad][pos + i];
                 buf ^= 1;
             }
             float *mine = reinterpret_cast<float *>(&bsh[warp][quad][0]) + pos;
             __syncwarp();  // every lane has read the previous beta
 #pragma unroll
-            for (int i = 0; i < 3; i++) {
+            for (int i = 0; i < NX; i++) {
                 own[i] -= x[i];
                 mine[i] = own[i];
             }
@@ -356,17 +379,27 @@ __global__ void __launch_bounds__(32 * NW, kResWarps / NW) k_refit_resident(
             }
         }
         // coefficients in the basis (1, x, y, x^2, y^2, x y): R^-1 beta (R^-1
-        // upper triangular), plus y_0 in the constant; groups 0 .. 5 make one
-        // each for their four pixels
-        if (coef && grp < 6) {
+        // upper triangular), plus y0 in the constant.  A pixel's rows i and 5 - i
+        // of R^-1 are one task, 12 a quad, dealt to the groups; FP32 values widened
+        // by bits: FP64 operations set the pace of short series (1024^2, 6 frames,
+        // no steps, 16 pixels a warp: six groups with a row of four pixels each
+        // 282 us, the tasks 182)
+        if (coef) {
+            for (int task = grp; task < 12; task += G) {
+                const int i = task % 3, j = task / 3;
+                const int64_t pj = p + j * STEP;
+                if (pj >= P) continue;
+                const float *b = reinterpret_cast<const float *>(&bsh[warp][quad][0]) + j;  // -beta_k at b[4 k]
+                const float origin = j == 0 ? y0[0] : j == 1 ? y0[1] : j == 2 ? y0[2] : y0[3];
+                double lo = i == 0 ? widen(origin) : 0.0, hi = 0.0;
 #pragma unroll
-            for (int j = 0; j < 4; j++) {
-                if (!live[j]) continue;
-                double c = grp == 0 ? (double)y0[j] : 0.0;
-#pragma unroll
-                for (int k = 0; k < 6; k++)
-                    if (k >= grp) c -= Rinv[grp * 6 + k] * (double)nb[k][j].x;
-                coef[(size_t)(p + j * STEP) * 6 + grp] = (float)c;
+                for (int k = 0; k < 6; k++) {
+                    const double v = widen(b[4 * k]);
+                    if (k > 1 || k >= i) lo -= rsh[i * 6 + k] * v;
+                    if (k > 4 || (k > 2 && k >= 5 - i)) hi -= rsh[(5 - i) * 6 + k] * v;
+                }
+                coef[(size_t)pj * 6 + i] = (float)lo;
+                coef[(size_t)pj * 6 + 5 - i] = (float)hi;
             }
         }
     }
@@ -511,7 +544,18 @@ Resident resident(bool vec) {
 // CTAs of 12 warps fit an SM's shared memory: longer runs per thread mean fewer
 // sums to exchange (T = 203: 2 warps 285 us, 8 warps 317 us).  Past 1152 frames
 // two such CTAs no longer fit with 16 pixels.
-Resident pick_resident(int64_t T, bool vec) {
+//
+// Short series: a block costs its exchanges and latencies whatever its frames,
+// so a warp takes 32 or 64 pixels instead of 16 where the image still gives
+// every CTA a block.  1024^2, 4 and 10 steps, 16 / 32 / 64 pixels: 6 frames
+// 256, 169, 136 and 376, 233, 174 us; 32 frames 327, 255, 230 and 488, 379,
+// 334; 48 frames 393, 313, 299 and 596, 482, 447; 96 frames 601, 523 and 928,
+// 818.  64^2, 16 / 32 pixels: 32 frames 52, 45 and 52, 49; 96 frames 56, 56 and
+// 60, 63.
+Resident pick_resident(int64_t T, int64_t P, bool vec) {
+    constexpr int64_t ctas = 152 * kResWarps;  // of one warp, at once
+    if (T <= 32 && P >= 64 * ctas) return resident<1, 16>(vec);
+    if (T <= 48 || (T <= 96 && P >= 32 * ctas)) return resident<1, 8>(vec);
     if (T <= 176) return resident<1, 4>(vec);
     if (T <= 352) return resident<2, 4>(vec);
     if (T <= 528) return resident<3, 4>(vec);
@@ -531,7 +575,7 @@ int launch_refit(const RefitArgs &a, char *err, size_t errlen) {
     cudaError_t e = cudaSuccess;
     if (a.T <= kRefitMaxResident) {
         const bool vec = P % 4 == 0 && (uintptr_t)a.data % 16 == 0 && (uintptr_t)a.resid % 16 == 0;
-        const Resident r = pick_resident(a.T, vec);
+        const Resident r = pick_resident(a.T, P, vec);
         const int groups = 32 * r.nw / r.quads, np = (int)((a.T + 2 * groups - 1) / (2 * groups));
         const size_t smem = (size_t)np * (2 * 32 * r.nw + 3 * groups) * sizeof(float4);
         e = cudaFuncSetAttribute(r.kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemAllowStatic);

@@ -154,3 +154,16 @@ def test_refit_outlier_in_an_end_frame(mf, T, outlier, frame):
     err = np.abs(R.cpu().numpy().astype(np.float64) - Ro)[rest].max(axis=0)
     tol = np.where(gone, 2e-6 * max(1.0, float(np.abs(D[rest]).max())), 2e-6 * float(np.abs(D).max()))
     assert (err <= tol).all(), "residual max err / bound %.3g" % (err / tol).max()
+
+
+@pytest.mark.parametrize("T,H,W", [
+    (6, 344, 340), (15, 350, 337), (32, 344, 340), (33, 350, 337),  # 64 pixels to a warp, and past them
+    (49, 245, 239), (96, 244, 240), (97, 245, 239),                 # 32 pixels, and past them
+    (48, 7, 9), (49, 7, 9),
+])
+def test_refit_short_series(mf, T, H, W):
+    # few frames: a warp takes more pixels where the image has enough of them;
+    # pixel counts that allow 128-bit rows and ones that do not, blocks past the
+    # grid's
+    from paper_2209_09848_gb300 import synth
+    _check(mf, synth.background_case(T, H, W, seed=T, n=5), 1.345, 3)
