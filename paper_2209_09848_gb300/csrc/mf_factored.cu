@@ -327,7 +327,14 @@ __device__ __forceinline__ bool fac_tile(const CUtensorMap &ymap, const FacParam
     // units of 32 rows x 16 columns, an item per lane.  Warps take the two
     // frames alternately, the last warps first (those past the column passes'
     // have no other work): a warp's frame, rows and columns are the same in
-    // every pair but for windows of more units than half the warps.
+    // every pair but for windows of more units than half the warps.  Tiles of 64
+    // columns (four units to 32 rows) pack the rows past the last 32: theirs are
+    // classes of one trajectory, 68 rows in a CTA of 20 warps, whose row pass is
+    // most of the work and took two rounds for 12 units a frame where 9 fit in
+    // one (500 x 300 x 700, 20 velocities on a line, FP32 2839 -> 2483 us, bf16
+    // 2966 -> 2570; items dealt to threads 2825 and 2850).  On 32 columns it
+    // costs the bf16 fine grid 2.5 %.
+    constexpr bool kPack = NI > 2;
     const int row_e = (nwarps - 1 - warp) & 1, row_u = (nwarps - 1 - warp) >> 1, row_n = nwarps >> 1;
     auto row_pair = [&](int f0, uint32_t rec0, uint32_t w0, uint32_t w1, uint32_t h0, bool two) {
         if (row_e && !two) return;
@@ -335,8 +342,14 @@ __device__ __forceinline__ bool fac_tile(const CUtensorMap &ymap, const FacParam
         const uint32_t hb = h0 + (row_e ? (uint32_t)(BH * HP * 4) : 0u);
         const float2 ph = lds2(hd + 8);  // FacHdr.cofs, nrows
         const int rows = __float_as_int(ph.y) - p.dth, cofs = __float_as_int(ph.x);
-        for (int u = row_u; 32 * (u / NI) < rows; u += row_n) {
-            const int m = u % NI, row = (u / NI) * 32 + lane;
+        const int whole = (rows >> 5) * NI;  // units of whole blocks
+        for (int u = row_u; kPack ? u < whole + (((rows & 31) * NI + 31) >> 5) : 32 * (u / NI) < rows; u += row_n) {
+            int m = u % NI, row = (u / NI) * 32 + lane;
+            if (kPack && u >= whole) {
+                const int it = (u - whole) * 32 + lane;
+                m = it % NI;
+                row = (rows & ~31) + it / NI;
+            }
             const float4 ua = lds4(hd + 16), ub = lds4(hd + 32);  // u_x; u_x(2), 1 / nrows, phase of 16-bit windows
             if (row >= rows) break;  // the last rows: no later unit has more of this lane's
             const uint32_t src = win + (uint32_t)(row * RP + kFacItem * m) * (uint32_t)sizeof(E);

@@ -572,3 +572,26 @@ def test_tile_rows_fit_the_image(mf, oracle, T, H, W, grid, vmax, segments):
         sh, tp = oracle.trajectory_table(vx, vy, T)
         N, D = oracle.search_full(c["res"], oracle.inverse_variance(c["sigma"], c["mask"]), sh, tp)
         check_search(*a, N, D, oracle, label="%s %s" % ((H, W), grid))
+
+
+@pytest.mark.parametrize("T,H,W,tile_h", [(33, 61, 70, 32), (18, 130, 129, 64), (9, 65, 64, 64), (21, 40, 200, 96)])
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_velocities_on_a_line(mf, oracle, T, H, W, tile_h, dtype):
+    # one trajectory to a class of v_x, tiles of 64 columns: windows of whole
+    # blocks of 32 rows and of a few rows more
+    from paper_2209_09848_gb300 import synth
+    c = synth.small_case(T, H, W, H + W, mask_frac=0.01, movers=2)
+    vx, vy = np.linspace(-0.3, 0.3, 6), np.linspace(0.2, -0.1, 6)
+    table = mf.prf_table_create(vx, vy, T, kernel=2, tile_w=64, tile_h=tile_h)
+    assert table.info()["groups"] == 6
+    sh, tp = oracle.trajectory_table(vx, vy, T)
+    lam = oracle.inverse_variance(c["sigma"], c["mask"])
+    if dtype == "f32":
+        N, D = oracle.search_full(c["res"], lam, sh, tp)
+        smax, amax, sall = _run(mf, c["res"], c["sigma"], c["mask"], table)
+    else:
+        deq = torch.from_numpy(c["res"]).to(torch.bfloat16).float().numpy()
+        y16, beta = oracle.weighted_stack16(deq, c["sigma"], c["mask"], None, "bf16")
+        N, D = oracle.search_weighted(y16, beta, lam, sh, tp)
+        smax, amax, sall = _run(mf, deq, c["sigma"], c["mask"], table, dtype=torch.bfloat16)
+    check_search(smax, amax, sall, N, D, oracle, label="%s %s" % ((H, W), tile_h))
