@@ -180,7 +180,9 @@ typedef struct {
                             warp out refills the stage, -1 = default */
     int32_t kernel;      /* 0 automatic, 1 general, 2 factored */
     int32_t group;       /* factored: trajectories per CTA, 0 = automatic */
-    int32_t tile_h;      /* factored: output rows per CTA, 0 = automatic */
+    int32_t tile_h;      /* factored: output rows per CTA, 0 = automatic (then
+                            mf_search takes shorter tiles on images so small that
+                            all of these still run at once) */
     int32_t tile_w;      /* factored: output columns per CTA, 0 = automatic */
     int32_t stages;      /* factored: frame windows in flight, 0 = automatic */
     int32_t segments;    /* factored: time segments, 0 = automatic (see below) */
@@ -447,6 +449,8 @@ mf_status mf_detect_workspace_size(int64_t H, int64_t W, int32_t max_out, size_t
  *            largest z, ordered by z rounded to FP32 descending, then flat
  *            index ascending (max_out 0..16384; 0 only counts);
  *   n_out    device int32[2]: detections found, detections written.
+ * A score that is not finite, or dwarfs the others, counts in the windows that
+ * hold it and nowhere else (z is 0 where a window's sums are not finite).
  * Asynchronous on `stream`; allocates nothing.  A union-find step that runs
  * past its iteration budget records code 3 in the status word read by
  * mf_device_status and leaves that pixel's detection incomplete.

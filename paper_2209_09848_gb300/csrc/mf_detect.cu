@@ -680,7 +680,8 @@ int launch_detect(const DetectArgs &a, char *err, size_t errlen) {
             snprintf(err, errlen, "cudaFuncSetAttribute(k_det_rows): %s", cudaGetErrorString(e));
             return (int)e;
         }
-        // below this an FP32 z (good to 1e-6) cannot belong to a candidate
+        // below this an FP32 z (the pairs' error, as it stands in z_out, is under
+        // 1e-6 of it) cannot belong to a candidate
         const double low = a.threshold - 1e-5 * std::max(1.0, std::fabs(a.threshold));
         const float thr_low = (float)std::max(-3e38, std::min(3e38, low));
         Scope sc(kKDetStats, stream);

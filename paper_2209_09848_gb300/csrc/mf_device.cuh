@@ -98,7 +98,9 @@ __device__ __forceinline__ void bulk_load(uint32_t dst, const void *src, uint32_
 // Programmatic dependent launches: a kernel lets the next one in its stream
 // start once all its CTAs have (or have ended), and a kernel waits for the one
 // before it to have completed, with everything it wrote.  Without that launch
-// attribute both do nothing.
+// attribute both do nothing.  Two reads of a search come without a wait of
+// their own: lambda in k_den_box and the weighted stack in a factored
+// numerator's later segments (see enqueue_den and start_early).
 __device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void wait_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 

@@ -46,11 +46,6 @@ namespace {
 
 using namespace dev;
 
-// The work of one CTA on one (output tile, trajectory group) of one search;
-// false if it gave up (a bounded wait ran out; the device status word says
-// why).  The CTA may have more warps than the search's layout uses (batched
-// searches share one launch): the extra warps take part in the row pass and
-// the barriers only.  `smem` is the CTA's 1024-aligned dynamic shared memory.
 // Shared memory by 32-bit address: the frame loop keeps its addresses in
 // registers, where C++ pointers into the dynamic array are formed again at every
 // access (with the row pass's fixed units below, 2.54e9 -> 2.35e9 instructions
@@ -177,6 +172,14 @@ __device__ __forceinline__ bool fac_locate(const FacParams &p, int tw, long long
     return true;
 }
 
+// The work of one CTA on one (output tile, trajectory group) of one search;
+// false if it gave up (a bounded wait ran out; the device status word says
+// why).  The CTA may have more warps than the search's layout uses (batched
+// searches share one launch): the extra warps take part in the row pass and
+// the barriers only.  `smem` is the CTA's 1024-aligned dynamic shared memory.
+// EARLY: a search's own launch, whose later segments wait for the one before in
+// the epilogue (see start_early).
+//
 // QG: the phase-plane form (phase-quantised banks, five taps, FP32 stacks):
 // per frame the row pass, then one column pass per rounded y-phase present
 // (a plane over the whole window), then one add per (trajectory, pixel)
@@ -350,7 +353,7 @@ __device__ __forceinline__ bool fac_tile(const CUtensorMap &ymap, const FacParam
                 m = it % NI;
                 row = (rows & ~31) + it / NI;
             }
-            const float4 ua = lds4(hd + 16), ub = lds4(hd + 32);  // u_x; u_x(2), 1 / nrows, phase of 16-bit windows
+            const float4 ua = lds4(hd + 16), ub = lds4(hd + 32);  // u_x; u_x(2), unused, phase of 16-bit windows
             if (row >= rows) break;  // the last rows: no later unit has more of this lane's
             const uint32_t src = win + (uint32_t)(row * RP + kFacItem * m) * (uint32_t)sizeof(E);
             const uint32_t dst = hb + (uint32_t)(row * HP + kFacItem * m) * 4u;
@@ -609,7 +612,11 @@ __device__ __forceinline__ bool fac_tile(const CUtensorMap &ymap, const FacParam
 // stack, so the kernel before must have completed; a later segment follows
 // segment 0, which waited for it, and needs its predecessor only for the
 // numerator plane, in the epilogue.  What follows may start when every CTA is
-// here.
+// here: the wait stands before launch_dependents, because later segments load
+// the weighted stack, and k_den_box lambda, without a wait of their own.  What
+// orders them is that no kernel of the chain lets its successor start before
+// the stack's writer has completed (and every kernel ends after the one before
+// it, so a search that follows on the stream finds all of it done).
 __device__ __forceinline__ void start_early(const FacParams &p) {
     if (p.seg == 0) wait_previous();
     launch_dependents();

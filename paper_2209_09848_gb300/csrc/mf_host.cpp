@@ -682,7 +682,6 @@ bool fac_layouts(mf_prf_table *t, HostLayouts &out) {
             fh.cofs8 = (int32_t)(t->shifts[((size_t)k0 * T + f) * 2 + 0] - 2 - 8 * floor_div(
                                      t->shifts[((size_t)k0 * T + f) * 2 + 0] - 2, 8));
             fh.nrows = h.nrows;
-            fh.inv_nrows = 1.0f / (float)h.nrows;
             for (int a = 0; a < 5; a++) fh.ux[a] = (float)t->fx[((size_t)k0 * T + f) * 5 + a];
             // phase planes: the distinct column-pass taps among the slots
             // (one per rounded y-phase present), in order of first use

@@ -120,7 +120,7 @@ struct alignas(16) FacHdr {
     int32_t cofs;                // row-pass column of output column 0 (0..3)
     int32_t nrows;               // row-pass rows this frame needs
     float ux[5];                 // u_x(a), a = -2..2
-    float inv_nrows;             // 1 / nrows, rounded to FP32 (splits row-pass items)
+    int32_t pad0;
     int32_t cofs8;               // the same for a window starting at a multiple of 8 columns (0..7):
                                  // 16-bit stacks, whose TMA boxes start at 16-byte boundaries
     int32_t pad;

@@ -1,7 +1,8 @@
 // Device side of libmf: the matched-filter search of Ganapathi (2022),
 // Section 3.2 (Eq. 5 and the maximum over the filter bank), for sm_103a.
 //
-// Kernels, in launch order:
+// Kernels, in launch order (of a factored search, whose numerator is in
+// mf_factored.cu: the denominator after it):
 //   k_lambda       inverse variance lambda = (1 - m) / sigma^2 into a zero-
 //                  padded image (Section 3.2 noise model; clipped pixels and
 //                  pixels outside the frame weigh 0);
@@ -147,6 +148,8 @@ __global__ void k_weight(const TIn *__restrict__ r, int64_t fstride, int64_t rst
                          TOut *__restrict__ y, int64_t T, int64_t H, int64_t W, int64_t yp,
                          const unsigned int *lmax_bits, float *__restrict__ beta) {
     constexpr bool kHalfScaled = std::is_same<TOut, __half>::value;
+    // in this order: a general search's k_den_box starts from here and reads
+    // lambda, this kernel's input, without a wait of its own
     wait_previous();
     launch_dependents();
     const float lmax = kHalfScaled ? __uint_as_float(*lmax_bits) : 0.f;
@@ -827,6 +830,8 @@ int grid_for(int64_t n, int threads) {
 
 // ---------------------------------------------------------- profiling ---
 
+// k_select: k_sel_hist and k_sel_gather; k_compact: k_sel_refine; k_sort:
+// k_sel_rank (names that callers of mf_profile_read know).
 const char *kKernelNames[kKernelCount] = {"k_lambda",    "k_weight",      "k_denominator", "k_numerator",
                                           "k_finalize",  "k_select",      "k_rescore",     "k_compact",
                                           "k_sort",      "k_det_stats",   "k_det_cc",      "k_det_emit",
@@ -1001,14 +1006,19 @@ int enqueue_pre(const SearchArgs &a, bool early, cudaStream_t stream, char *err,
     return 0;
 }
 
-// The denominator; `early`: as a programmatic dependent of the numerator's last
-// launch.  It needs lambda only, complete since that numerator's first segment
-// waited for the weighted stack, so it takes the SMs the numerator's last CTAs
-// leave (a factored search needs 1 / sqrt(D) only at its finalisation).  With
-// that and every kernel of a factored search started early, 333 frames of 301 x
-// 277 pixels and 54 trajectories take 707 us instead of 783, 32 frames of 128 x
-// 128 and 16 trajectories 43.5 instead of 47.2; the general numerator's keys hold final SNR, so its
-// denominator comes first.  (For that numerator also a cleared key buffer.)
+// The denominator; `early`: k_den_box as a programmatic dependent of the kernel
+// before it, the numerator's last launch of a factored search, the weighting of
+// a general one (whose keys hold final SNR).  It reads lambda, through the L1
+// cache and without a wait: lambda's writer k_lambda, a launch in full order,
+// has completed before k_weight lets anything start (its wait stands before its
+// launch_dependents, and segment 0's of the numerator likewise), and no kernel
+// since has put lambda into an L1 cache.  A kernel put between them, or a
+// k_lambda started early, would have to keep that.  In a factored search the
+// denominator so takes the SMs that the numerator's last CTAs leave (1 / sqrt(D)
+// is needed only at the finalisation): with every kernel started early, 333
+// frames of 301 x 277 pixels and 54 trajectories take 707 us instead of 783, 32
+// frames of 128 x 128 and 16 trajectories 43.5 instead of 47.2.  (For the
+// general numerator also a cleared key buffer.)
 int enqueue_den(const SearchArgs &a, bool early, cudaStream_t stream, char *err, size_t errlen) {
     const mf_prf_table &tab = *a.tab;
     const WorkspaceLayout &L = a.L;
@@ -1065,7 +1075,6 @@ int enqueue_den(const SearchArgs &a, bool early, cudaStream_t stream, char *err,
     return 0;
 }
 
-// Tensor map over the weighted stack and the numerator's parameters.
 // Tile and staged window of the general numerator's CTAs.
 struct NumGeometry {
     int tw, th, S, BH;
@@ -1108,6 +1117,7 @@ bool numerator_halves(const Plan &pl, int64_t H, int64_t W) {
     return full > 152 || numerator_ctas(pl, g, H, W) <= 152;
 }
 
+// Tensor map over the weighted stack and the numerator's parameters.
 int numerator_params(const SearchArgs &a, const NumGeometry &geo, CUtensorMap *map, NumParams *np, int *tiles_y,
                      char *err, size_t errlen) {
     const mf_stack &st = *a.stack;
@@ -1330,7 +1340,7 @@ struct BatchDevice {
         int tw = 32;
         int etype = MF_F32;        // element type of the weighted stacks
         int seg = 0;               // time segment (groups run in segment order)
-        int first = 0, count = 0;  // range in d_fmaps / d_fitems
+        int first = 0, count = 0;  // range in d_fmaps and h_fitems
         long long total = 0;       // CTA work entries
         size_t smem = 0;
         int warps = 0;
@@ -1338,8 +1348,7 @@ struct BatchDevice {
     std::vector<FacGroup> fac;
     std::vector<int> item_chain;  // the chain of each search, -1: general numerator
     CUtensorMap *d_fmaps = nullptr;
-    FacBatchItem *d_fitems = nullptr;
-    std::vector<FacBatchItem> h_fitems;  // the same, passed by value to each launch
+    std::vector<FacBatchItem> h_fitems;  // passed by value to each launch
     unsigned long long *d_fcounters = nullptr;  // one per group
     CUtensorMap *d_maps = nullptr;
     BatchItem *d_items = nullptr;
@@ -1356,7 +1365,6 @@ void batch_free(BatchDevice *b) {
     cudaFree(b->d_items);
     cudaFree(b->d_counters);
     cudaFree(b->d_fmaps);
-    cudaFree(b->d_fitems);
     cudaFree(b->d_fcounters);
     for (int i = 0; i < BatchDevice::kSide; i++) {
         if (b->side[i]) cudaStreamDestroy(b->side[i]);
@@ -1458,13 +1466,10 @@ int batch_build(const SearchArgs *items, int n, BatchDevice **out, char *err, si
     }
     cudaError_t e = cudaSuccess;
     if (!fitems.empty()) e = cudaMalloc((void **)&b->d_fmaps, fmaps.size() * sizeof(CUtensorMap));
-    if (e == cudaSuccess && !fitems.empty()) e = cudaMalloc((void **)&b->d_fitems, fitems.size() * sizeof(FacBatchItem));
     if (e == cudaSuccess && !fitems.empty())
         e = cudaMalloc((void **)&b->d_fcounters, b->fac.size() * sizeof(unsigned long long));
     if (e == cudaSuccess && !fitems.empty())
         e = cudaMemcpy(b->d_fmaps, fmaps.data(), fmaps.size() * sizeof(CUtensorMap), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess && !fitems.empty())
-        e = cudaMemcpy(b->d_fitems, fitems.data(), fitems.size() * sizeof(FacBatchItem), cudaMemcpyHostToDevice);
     b->h_fitems = fitems;
     int dev = 0;
     if (e == cudaSuccess) e = cudaGetDevice(&dev);
