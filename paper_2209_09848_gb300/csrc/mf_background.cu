@@ -64,7 +64,7 @@ size_t align256(size_t x) { return (x + 255) / 256 * 256; }
 // with three register operands run at three quarters of the pipe's rate here,
 // and the clip's min / max are half rate -- and the whole step 50, the rest
 // being the exchanges, the barrier and three warps a scheduler to cover them.
-// 1000 x 2048^2, 10 steps: 63.7 -> 41.4 ms; 203 x 317 x 411: 488 -> 287 us.
+// 1000 x 2048^2, 10 steps: 63.7 -> 41.8 ms; 203 x 317 x 411: 488 -> 289 us.
 // Rows of 16 pixels (two whole sectors) because 32-pixel rows leave one CTA an
 // SM and 8-pixel rows double the requests (the load alone: 3.3 against 6.5 ms
 // at 1000 x 1024^2).  Values in registers (24 frames a thread, T = 1000): 38.9
